@@ -30,6 +30,7 @@ struct TcArgs {
   unsigned int* err;              // device error word
   // split-K (few output tiles): the k range of a tile is cut into ksplit parts on different CTAs
   int ksplit;                     // set by the launcher (1: no split)
+  int rows_first;                 // set by the launcher: row blocks move fastest over the tiles
   void* partials;                 // tc_split_partial_bytes(M) bytes of workspace
   unsigned int* tile_counters;    // one per output tile, zero between calls
 };
