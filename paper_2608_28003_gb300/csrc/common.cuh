@@ -184,6 +184,20 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
     if (clock64() - t0 > budget) return false;
   return true;
 }
+// The same for a whole warp: the result, and so the control flow that depends on it, is uniform.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, long long budget) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const long long t0 = clock64();
+  while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity)))
+    if (__any_sync(0xffffffffu, clock64() - t0 > budget)) return false;
+  return true;
+}
+// One lane of a converged warp, the same one every time.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+  return r != 0;
+}
 // Start fetching a tensor map (a kernel parameter) so the first copy does not wait for it.
 __device__ __forceinline__ void prefetch_tmap(const void* tmap) {
   asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");
@@ -281,6 +295,92 @@ __device__ __forceinline__ float gelu_tanh_recipe(float g) {
 }
 
 __device__ __forceinline__ float geglu_recipe(float g, float u) { return __fmul_rn(gelu_tanh_recipe(g), u); }
+
+// Two fp32 values in one 64-bit register: each half of a packed operation is one IEEE operation,
+// rounded to nearest even.  A packed multiply feeding a packed add is contracted into one fused
+// operation whatever the rounding modifier says, so f2_mul adds a -0 that the compiler cannot know
+// (f2_neg_zero: gridDim.z is 1 in every launch); a b + (-0) is the rounded product, signs included.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 f2_pack(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};\n" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;\n" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 f2_both(uint32_t bits) { return ((f32x2)bits << 32) | bits; }
+__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+__device__ __forceinline__ f32x2 f2_neg_zero() { return f2_both(0x7fffffffu + gridDim.z); }
+__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b, f32x2 neg_zero) { return f2_fma(a, b, neg_zero); }
+
+// Whether geglu_pair takes this gate: 2^-60 <= |g| <= 2^60 or +0 (an INT32 sum of 0); NaN, infinities
+// and -0 are left to geglu_recipe.
+__device__ __forceinline__ bool geglu_in_range(float g) {
+  const uint32_t b = __float_as_uint(g);
+  return (b & 0x7fffffffu) - 0x21800000u <= 0x5d800000u - 0x21800000u || b == 0u;
+}
+
+// geglu_recipe of two (gate, up) pairs, bit for bit, for gates in range: packed operations and no
+// branch.  The recipe's division compiles to a routine with a branch to a slow path for extreme
+// operands (1 + 2^w reaches 2^126), so neighbouring elements could not be interleaved and the GeGLU
+// epilogue, not the MMAs, bounded the GEMM: 2048 x 1152 -> 13824 W8A8 69 us (50 us without GeGLU),
+// now 52; bf16 52.9 -> 45.8.
+// What makes the steps below the recipe's:
+//  * rint(w) is the fp32 sum w + 1.5 2^23 less 1.5 2^23 (|w| < 2^22, ties to even), whose low
+//    mantissa bits are the integer;
+//  * w is clamped at -60 instead of -126: 1 + 2^w rounds to 1 either way;
+//  * everything from 2^w on is scaled by 2^-64 (exact: no step leaves the normal range), which keeps
+//    the reciprocal of 1 + 2^w normal;
+//  * the quotient is correctly rounded by Markstein's method (Computation of elementary functions
+//    on the IBM RISC System/6000, 1990): a reciprocal within one ulp, corrected once by its exact
+//    residual, then the quotient corrected by its own exact residual.
+__device__ __forceinline__ void geglu_pair(float g0, float g1, float u0, float u1, f32x2 nz, float& h0, float& h1) {
+  const f32x2 magic = f2_both(0x4b400000u), minus1 = f2_both(0xbf800000u), tiny = f2_both(0x1f800000u);  // 2^-64
+  const f32x2 g = f2_pack(g0, g1);
+  const f32x2 g3 = f2_mul(f2_mul(g, g, nz), g, nz);
+  const f32x2 t = f2_add(g, f2_mul(f2_both(0x3d372713u), g3, nz));
+  const f32x2 w2 = f2_mul(f2_both(0xc038aa3bu), f2_mul(f2_both(0x3f4c422au), t, nz), nz);
+  float wa, wb;
+  f2_unpack(w2, wa, wb);
+  wa = fminf(fmaxf(wa, -60.0f), 126.0f);
+  wb = fminf(fmaxf(wb, -60.0f), 126.0f);
+  const f32x2 w = f2_pack(wa, wb);
+  const f32x2 shifted = f2_add(w, magic);
+  const f32x2 f = f2_add(w, f2_fma(shifted, minus1, magic));  // w - rint(w)
+  f32x2 p = f2_both(0x377fe5feu);
+  p = f2_add(f2_mul(p, f, nz), f2_both(0x39218489u));
+  p = f2_add(f2_mul(p, f, nz), f2_both(0x3aaec3ffu));
+  p = f2_add(f2_mul(p, f, nz), f2_both(0x3c1d955bu));
+  p = f2_add(f2_mul(p, f, nz), f2_both(0x3d635847u));
+  p = f2_add(f2_mul(p, f, nz), f2_both(0x3e75fdf0u));
+  p = f2_add(f2_mul(p, f, nz), f2_both(0x3f317218u));
+  p = f2_add(f2_mul(p, f, nz), f2_both(0x3f800000u));
+  float sa, sb;
+  f2_unpack(shifted, sa, sb);
+  const f32x2 scale = f2_pack(__uint_as_float((__float_as_uint(sa) << 23) + (63u << 23)),
+                              __uint_as_float((__float_as_uint(sb) << 23) + (63u << 23)));  // 2^(n - 64)
+  const f32x2 d = f2_add(tiny, f2_mul(p, scale, nz)), nd = f2_mul(d, minus1, nz);
+  float da, db, ya, yb;
+  f2_unpack(d, da, db);
+  asm("rcp.approx.ftz.f32 %0, %1;\n" : "=f"(ya) : "f"(da));
+  asm("rcp.approx.ftz.f32 %0, %1;\n" : "=f"(yb) : "f"(db));
+  f32x2 y = f2_pack(ya, yb);
+  y = f2_fma(y, f2_fma(nd, y, f2_both(0x3f800000u)), y);
+  f32x2 q = f2_mul(g, y, nz);
+  q = f2_fma(f2_fma(nd, q, g), y, q);
+  f2_unpack(f2_mul(f2_mul(q, tiny, nz), f2_pack(u0, u1), nz), h0, h1);
+}
 
 // ------------------------------------------------------------------------- reductions
 __device__ __forceinline__ float warp_max(float v) {

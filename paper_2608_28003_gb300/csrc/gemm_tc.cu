@@ -52,6 +52,8 @@ __host__ __device__ constexpr int bk_elems(int mode) { return mode == kModeFp8 ?
 __host__ __device__ constexpr int elem_bytes(int mode) { return mode == kModeFp8 ? 1 : 2; }
 constexpr int kEpiWarps = 16;                   // four per TMEM lane quarter: one per column quarter
 constexpr int kParts = kEpiWarps / 4;
+// 32-column groups of an epilogue warp on a tile of bn columns (of two groups, a warp has both or none)
+constexpr int tile_groups(int bn) { return (bn / 32 + kParts - 1) / kParts; }
 constexpr int kProdWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1;
 constexpr int kThreads = 32 * (kEpiWarps + 2);
 // The 512 epilogue threads test the rows once per kernel, while the first stages load: bit i of
@@ -118,20 +120,6 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
   return r;
 }
 
-// 32 consecutive fp32 values p[c0 .. c0 + 31] into w, 0 past n (c0 a multiple of 32, p 16-byte
-// aligned): eight 16-byte loads when the group lies inside n.  Every lane of a warp reads the same
-// addresses (a broadcast).
-
-// The dequantising epilogue of one 32-column group: w holds s_w of the columns on entry and
-// fl(fl(s_x s_w) acc) (+ bias) on exit (Eq. gemm-final); acc is the INT32 sum (W8A8) or the fp32
-// one (FP8).
-template <typename T>
-__device__ __forceinline__ float acc_as_f32(T v);
-template <>
-__device__ __forceinline__ float acc_as_f32<int>(int v) { return __int2float_rn(v); }
-template <>
-__device__ __forceinline__ float acc_as_f32<uint32_t>(uint32_t v) { return __uint_as_float(v); }
-
 // Column values of the epilogue (s_w, bias) one column per lane: lane j holds column c0 + j of
 // each of the warp's NG groups, loaded at the start of a tile, before the wait for its
 // accumulator, so that the load latency overlaps the MMAs; element j of a group takes its values
@@ -145,30 +133,20 @@ __device__ __forceinline__ void load_colvals(const TcArgs& a, bool want_sw, int 
                                              ColVals<NG>& cv) {
 #pragma unroll
   for (int i = 0; i < NG; ++i) {
-    const int c = n0 + 32 * (part + kParts * i) + lane;
-    const bool in = 32 * (part + kParts * i) < bn && c < a.N;
+    const int c = n0 + 32 * (NG * part + i) + lane;
+    const bool in = 32 * (NG * part + i) < bn && c < a.N;
     cv.sw[i] = want_sw && in ? __ldg(a.s_w + c) : 0.0f;
     cv.b[i] = a.bias && in ? __ldg(a.bias + c) : 0.0f;
   }
 }
-// fl(fl(s_x s_w) acc) (+ bias) of one 32-column group (Eq. gemm-final); acc is the INT32 sum
-// (W8A8) or the fp32 one (FP8); sw / b are this lane's column values of the group.
-// Two IEEE fp32 products, each rounded to nearest even (the packed form of two __fmul_rn).
-__device__ __forceinline__ void fmul2_rn(float a0, float a1, float b0, float b1, float& d0, float& d1) {
-  const unsigned long long x = ((unsigned long long)__float_as_uint(a1) << 32) | __float_as_uint(a0);
-  const unsigned long long y = ((unsigned long long)__float_as_uint(b1) << 32) | __float_as_uint(b0);
-  unsigned long long z;
-  asm("mul.rn.f32x2 %0, %1, %2;\n" : "=l"(z) : "l"(x), "l"(y));
-  d0 = __uint_as_float((uint32_t)z);
-  d1 = __uint_as_float((uint32_t)(z >> 32));
-}
-template <typename T>
-__device__ __forceinline__ void dequant32(bool has_bias, float sx, float sw, float b, const T* acc, float (&v)[32]) {
+// fl(fl(s_x s_w) acc) (+ bias) of one 32-column group (Eq. gemm-final); v holds acc on entry, the
+// INT32 sum as fp32 (W8A8) or the fp32 sum (FP8); sw / b are this lane's column values of the group.
+__device__ __forceinline__ void dequant32(bool has_bias, float sx, float sw, float b, f32x2 nz, float (&v)[32]) {
+  const f32x2 sx2 = f2_pack(sx, sx);
 #pragma unroll
   for (int j = 0; j < 32; j += 2) {
-    float t0, t1;
-    fmul2_rn(sx, sx, __shfl_sync(0xffffffffu, sw, j), __shfl_sync(0xffffffffu, sw, j + 1), t0, t1);
-    fmul2_rn(t0, t1, acc_as_f32<T>(acc[j]), acc_as_f32<T>(acc[j + 1]), v[j], v[j + 1]);
+    const f32x2 s2 = f2_mul(sx2, f2_pack(__shfl_sync(0xffffffffu, sw, j), __shfl_sync(0xffffffffu, sw, j + 1)), nz);
+    f2_unpack(f2_mul(s2, f2_pack(v[j], v[j + 1]), nz), v[j], v[j + 1]);
     if (has_bias) {
       v[j] = __fadd_rn(v[j], __shfl_sync(0xffffffffu, b, j));
       v[j + 1] = __fadd_rn(v[j + 1], __shfl_sync(0xffffffffu, b, j + 1));
@@ -181,14 +159,13 @@ __device__ __forceinline__ void add_bias32(float b, float (&v)[32]) {
 }
 
 // ------------------------------------------------------------------ epilogue through TMA stores
-// Each epilogue warp stages 32 rows x 32 columns of output (its rows, one 32-column group) in its
-// 2 KB shared-memory block and one lane stores the block with a 2-D TMA store (rows past M and
-// columns past N are clipped by the tensor map), so the global writes are whole rows, not one
-// 16-byte piece per thread and row; the warp waits for the store to have read the block before it
-// refills it (the other warps of its sub-partition issue meanwhile).  A staged row is 64 bytes (32 bf16 or 16 fp32: fp32 output goes
-// out as two blocks of 16 columns) or 32 (GeGLU); the block is kept in the tensor map's swizzled
-// layout of that width (16-byte chunk c of row r at chunk c ^ ((r >> 1) & 3), or c ^ ((r >> 2) & 1)),
-// so the 16-byte stores of eight consecutive rows fall in eight different bank groups.
+// An epilogue warp stages its 32 rows in its 2 KB shared-memory block and one lane stores the block
+// with a 2-D TMA store (rows past M and columns past N are clipped by the tensor map): bf16 a
+// 32-column group at a time (64-byte rows), GeGLU all of the warp's groups of a tile (64- or 32-byte
+// rows), fp32 logits 16 rows of a group at a time (whole 128-byte lines).  16-byte chunk c of row r
+// sits at chunk c ^ (r & 7), c ^ ((r >> 1) & 3) or c ^ ((r >> 2) & 1), the tensor map's swizzle of
+// that width, so eight consecutive rows fall in different banks.  (Stores from registers, 32 bytes
+// per thread, took 360 us on the 509-token lm_head against 245: each spreads over 32 lines.)
 
 __device__ __forceinline__ void fence_proxy_async_shared() {
   asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -203,77 +180,187 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 __device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
 
-// The epilogue of 32 consecutive columns col0 .. col0+31 of this thread's row (lane of the warp
-// whose rows start at row0): bf16 output, GeGLU of the interleaved gate/up columns (two 16-column
-// blocks: 8 gate, then the 8 matching up channels), or fp32 logits with the row's running top-1 key.
-__device__ __forceinline__ void stage_cols32(const TcArgs& a, const CUtensorMap* tmY, uint32_t buf,
-                                             int row0, int col0, int lane, const float (&v)[32], bool want_top,
-                                             unsigned long long& best) {
-  const int row = row0 + lane;
-  if (a.kind == EPI_F32 && want_top && row < a.M) {
+// Running top-1 of a row: the best key this thread has seen in the tile, and the largest logit
+// known for the row (from this tile or, at its start, from the keys every CTA reduces into).
+struct Top {
+  float known;
+  unsigned long long best;
+};
+// The value behind a key's upper half (the inverse of float_order_key); NaN for the empty key.
+__device__ __forceinline__ float key_value(unsigned long long key) {
+  const uint32_t k = (uint32_t)(key >> 32);
+  return __uint_as_float((k & 0x80000000u) ? k ^ 0x80000000u : ~k);
+}
+// max that is NaN when an operand is
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;\n" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
+// Chunks at .. at + n - 1 of this lane's row, kChunks 16-byte chunks wide, into the warp's block.
+template <int kChunks, int n>
+__device__ __forceinline__ void stage_row(uint32_t buf, int r, int at, const uint32_t* w) {
+  const uint32_t sw = kChunks == 8 ? (uint32_t)(r & 7) : kChunks == 4 ? (uint32_t)((r >> 1) & 3) : (uint32_t)((r >> 2) & 1);
+  const uint32_t dst = buf + (uint32_t)(r * kChunks * 16);
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const int col = col0 + j;
-      if (col < a.N) {
-        const unsigned long long key =
-            ((unsigned long long)float_order_key(v[j]) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)col);
-        best = key > best ? key : best;
-      }
-    }
-  }
-  if (a.kind == EPI_F32) {
-    if (!a.logits) return;  // top-1 only
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (lane == 0) bulk_wait_read0();  // the previous store has read the block
-      __syncwarp();
-      const uint32_t dst = buf + (uint32_t)(lane * 64), sw = (uint32_t)((lane >> 1) & 3);
-#pragma unroll
-      for (int j4 = 0; j4 < 4; ++j4)
-        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst + 16 * ((uint32_t)j4 ^ sw)),
-                     "f"(v[16 * h + 4 * j4]), "f"(v[16 * h + 4 * j4 + 1]), "f"(v[16 * h + 4 * j4 + 2]),
-                     "f"(v[16 * h + 4 * j4 + 3])
-                     : "memory");
-      fence_proxy_async_shared();
-      __syncwarp();
-      if (lane == 0) {
-        tma_store_2d(tmY, buf, col0 + 16 * h, row0);
-        bulk_commit();
-      }
-    }
-    return;
-  }
-  if (lane == 0) bulk_wait_read0();  // the previous store has read the block
+  for (int c = 0; c < n; ++c)
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst + 16 * ((uint32_t)(at + c) ^ sw)), "r"(w[4 * c]),
+                 "r"(w[4 * c + 1]), "r"(w[4 * c + 2]), "r"(w[4 * c + 3])
+                 : "memory");
+}
+// Before the block is refilled: the previous store has read it.
+__device__ __forceinline__ void block_free(int lane) {
+  if (lane == 0) bulk_wait_read0();
   __syncwarp();
-  if (a.kind == EPI_GEGLU) {
-    uint32_t w[8];
-#pragma unroll
-    for (int hq = 0; hq < 2; ++hq)
-#pragma unroll
-      for (int j = 0; j < 8; j += 2)
-        w[4 * hq + j / 2] = pack_bf16x2(geglu_recipe(v[16 * hq + j], v[16 * hq + 8 + j]),
-                                        geglu_recipe(v[16 * hq + j + 1], v[16 * hq + 9 + j]));
-    const uint32_t dst = buf + (uint32_t)(lane * 32), sw = (uint32_t)((lane >> 2) & 1);
-    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst + 16 * sw), "r"(w[0]), "r"(w[1]), "r"(w[2]),
-                 "r"(w[3])
-                 : "memory");
-    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst + 16 * (1u ^ sw)), "r"(w[4]), "r"(w[5]),
-                 "r"(w[6]), "r"(w[7])
-                 : "memory");
-  } else {
-    const uint32_t dst = buf + (uint32_t)(lane * 64), sw = (uint32_t)((lane >> 1) & 3);
-#pragma unroll
-    for (int j8 = 0; j8 < 4; ++j8)
-      asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst + 16 * ((uint32_t)j8 ^ sw)),
-                   "r"(pack_bf16x2(v[8 * j8], v[8 * j8 + 1])), "r"(pack_bf16x2(v[8 * j8 + 2], v[8 * j8 + 3])),
-                   "r"(pack_bf16x2(v[8 * j8 + 4], v[8 * j8 + 5])), "r"(pack_bf16x2(v[8 * j8 + 6], v[8 * j8 + 7]))
-                   : "memory");
-  }
+}
+__device__ __forceinline__ void store_block(const CUtensorMap* tmY, uint32_t buf, int lane, int col, int row0) {
   fence_proxy_async_shared();
   __syncwarp();
   if (lane == 0) {
-    tma_store_2d(tmY, buf, a.kind == EPI_GEGLU ? col0 >> 1 : col0, row0);
+    tma_store_2d(tmY, buf, col, row0);
     bulk_commit();
+  }
+}
+
+// The row's running top-1 over logits v of columns col0 .. col0 + n - 1 (n <= 32).  Only a group whose
+// maximum reaches the largest logit known for the row can hold its top-1: a maximum of 32 values
+// instead of 32 64-bit keys (those are left to groups with NaN or columns past N).  bf16 lm_head at
+// 509 tokens: 248 -> 224 us.
+__device__ __forceinline__ void top_cols32(const float (&v)[32], int col0, int n, Top& top) {
+  float m[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) m[j] = max_nan(max_nan(v[j], v[j + 8]), max_nan(v[j + 16], v[j + 24]));
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+    for (int j = 0; j < o; ++j) m[j] = max_nan(m[j], m[j + o]);
+  const float mx = m[0];
+  if (mx < top.known) return;
+  if (mx == mx && n == 32) {  // the lowest column that holds the maximum
+    int at = 31;
+#pragma unroll
+    for (int j = 30; j >= 0; --j) at = v[j] == mx ? j : at;
+    const unsigned long long key = ((unsigned long long)float_order_key(mx) << 32) |
+                                   (unsigned long long)(0xFFFFFFFFu - (uint32_t)(col0 + at));
+    top.best = key > top.best ? key : top.best;
+    top.known = mx;
+    return;
+  }
+  float t[32];
+#pragma unroll
+  for (int j = 0; j < 32; ++j) t[j] = v[j];
+#pragma unroll 1
+  for (int j = 0; j < n; ++j) {
+    const unsigned long long key =
+        ((unsigned long long)float_order_key(t[j]) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)(col0 + j));
+    top.best = key > top.best ? key : top.best;
+  }
+  top.known = key_value(top.best);
+}
+
+// GeGLU of 32 interleaved gate/up columns (two blocks of 8 gate, then the 8 matching up channels) as
+// 16 bf16 values; live: the row is stored.
+__device__ __forceinline__ void geglu_cols32(const float (&v)[32], bool live, f32x2 nz, uint32_t* w) {
+  bool usual = true;  // every gate of the row in geglu_pair's range
+#pragma unroll
+  for (int hq = 0; hq < 2; ++hq)
+#pragma unroll
+    for (int j = 0; j < 8; j += 2) {
+      const float g0 = v[16 * hq + j], g1 = v[16 * hq + j + 1];
+      float h0, h1;
+      geglu_pair(g0, g1, v[16 * hq + 8 + j], v[16 * hq + 9 + j], nz, h0, h1);
+      w[4 * hq + j / 2] = pack_bf16x2(h0, h1);
+      usual = usual && geglu_in_range(g0) && geglu_in_range(g1);
+    }
+  if (!usual && live) {  // a loop, not 16 copies of the general recipe: the code stays in the caches
+    float t[32];
+    uint32_t x[8];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) t[j] = v[j];
+#pragma unroll 1
+    for (int j = 0; j < 8; ++j) {
+      const int c = 2 * j + ((2 * j) & 8);
+      x[j] = pack_bf16x2(geglu_recipe(t[c], t[c + 8]), geglu_recipe(t[c + 1], t[c + 9]));
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) w[j] = x[j];
+  }
+}
+
+// One finished tile of BN columns from n0: this warp's NG 32-column groups (group part NG + i) of its
+// 32 rows from row0, from the accumulator at tm (release() hands the slot back once the last group has
+// been read) or, folded, from the INT32 sums (a local array: in registers they would spill).  One copy of
+// the epilogue's code for the groups and both paths: unrolled, sixteen warps at different places in it
+// waited for instructions.
+template <int kMode, int BN, int NG, class Release>
+__device__ __forceinline__ void emit_tile(const TcArgs& a, const CUtensorMap* tmY, uint32_t buf, bool folded,
+                                          const int* sums, uint32_t tm, int row0, int n0, int part, int lane,
+                                          const ColVals<NG>& cv, float sx, bool want_top, f32x2 nz, Top& top,
+                                          Release release) {
+  constexpr bool kInt8 = kMode == kModeI8;
+  const int row = row0 + lane, c0 = n0 + 32 * NG * part;
+  if (32 * NG * part >= BN) {  // no group of this tile
+    if (!folded) release();
+    return;
+  }
+#pragma unroll 1
+  for (int i = 0; i < NG; ++i) {
+    float v[32];
+    if (!kInt8 || !folded) {
+      uint32_t r[32];
+      __syncwarp();
+      tmem_ld32(tm + (uint32_t)(32 * (NG * part + i)), r);
+      if (i == NG - 1) release();
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+      if (kInt8 && a.acc_dbg && row < a.M) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+          if (c0 + 32 * i + j < a.N) a.acc_dbg[(size_t)row * a.N + c0 + 32 * i + j] = __float2int_rn(v[j]);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        const int q = sums[32 * i + j];
+        if (a.acc_dbg && row < a.M && c0 + 32 * i + j < a.N) a.acc_dbg[(size_t)row * a.N + c0 + 32 * i + j] = q;
+        v[j] = __int2float_rn(q);
+      }
+    }
+    const float sw = i == 0 ? cv.sw[0] : cv.sw[NG - 1], b = i == 0 ? cv.b[0] : cv.b[NG - 1];
+    if constexpr (kMode != kModeBf16)
+      dequant32(a.bias != nullptr, sx, sw, b, nz, v);
+    else if (a.bias)
+      add_bias32(b, v);
+    if (a.kind == EPI_F32) {
+      if (want_top && row < a.M) top_cols32(v, c0 + 32 * i, min(32, a.N - c0 - 32 * i), top);
+      __syncwarp();
+      if (a.logits) {
+        uint32_t w[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) w[j] = __float_as_uint(v[j]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          block_free(lane);
+          if (lane / 16 == h) stage_row<8, 8>(buf, lane & 15, 0, w);
+          store_block(tmY, buf, lane, c0 + 32 * i, row0 + 16 * h);
+        }
+      }
+    } else if (a.kind == EPI_GEGLU) {
+      uint32_t w[8];
+      geglu_cols32(v, row < a.M, nz, w);
+      __syncwarp();
+      if (i == 0) block_free(lane);
+      stage_row<2 * NG, 2>(buf, lane, 2 * i, w);
+      if (i == NG - 1) store_block(tmY, buf, lane, c0 >> 1, row0);
+    } else {
+      uint32_t w[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) w[j] = pack_bf16x2(v[2 * j], v[2 * j + 1]);
+      block_free(lane);
+      stage_row<4, 4>(buf, lane, 0, w);
+      store_block(tmY, buf, lane, c0 + 32 * i, row0);
+    }
   }
 }
 
@@ -404,24 +491,35 @@ __global__ void __launch_bounds__(kThreads, 1)
   // Persistent: CTA b takes units b, b + grid, ... in the order of TileOrder.
   if (warp == kProdWarp) {
     // ---------------------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      bool ok = true;
-      int g = 0;  // stages issued
-      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
-        const int t = u / KS, n0 = ord.col(t) * BN, m0 = ord.row(t) * kBM;
-        const int kb_end = kb_hi(u);
-        for (int kb = kb_lo(u); kb < kb_end; ++kb, ++g) {
-          const int s = g % S;
-          if (!mbar_wait_bounded(empty0 + 8 * s, (uint32_t)(((g / S) & 1) ^ 1), kWaitBudgetCycles)) {
-            ok = false;
-            break;
-          }
-          const uint32_t bar = full0 + 8 * s;
+    // The whole warp walks the stages and an elected lane issues: the addresses and coordinates stay
+    // in uniform registers, which is where the copy and MMA instructions take them from.  Issued by
+    // one divergent lane, each instruction's operands were moved there first, and the MMAs waited for
+    // their issue: 2048 x 6912 -> 1152 bf16 39.6 -> 31.4 us, W8A8 44.7 -> 31.4.
+    bool ok = true;
+    int g = 0, s = 0;  // stages issued; the next one's slot and phase
+    uint32_t ph = 1;
+    for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+      const int t = u / KS, n0 = ord.col(t) * BN, m0 = ord.row(t) * kBM;
+      const int kb_end = kb_hi(u);
+      for (int kb = kb_lo(u); kb < kb_end; ++kb, ++g) {
+        if (!mbar_wait_warp(empty0 + 8 * s, ph, kWaitBudgetCycles)) {
+          ok = false;
+          break;
+        }
+        const uint32_t bar = full0 + 8 * s;
+        if (elect_one()) {
           mbar_arrive_expect_tx(bar, (uint32_t)(a_box_rows(a.M) * kSwz) + GG::BBytes);
           tma_load_2d(sA + (uint32_t)s * kABytes, &tmA, kb * BKe, m0, bar);
           tma_load_2d(sB + (uint32_t)s * GG::BBytes, &tmB, kb * BKe, n0, bar);
         }
+        __syncwarp();
+        if (++s == S) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
+    }
+    if (lane == 0) {
       if (!ok) atomicOr(a.err, DEVERR_PRODUCER_WAIT);
       for (int j = g > S ? g - S : 0; j < g; ++j) {  // let the last copies land before exit
         if (!mbar_wait_bounded(full0 + 8 * (j % S), (uint32_t)((j / S) & 1), kWaitBudgetCycles)) {
@@ -432,70 +530,76 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == kMmaWarp) {
     // ---------------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_f16(kMode == kModeBf16 ? 1u : 0u, BN, kBM);
-      bool ok = true, known = false;  // known: the epilogue's exactness scan has been read
-      uint32_t fail = 0u;
-      int g = 0, q = 0;  // stages consumed, accumulator chunks produced
-      // One accumulator slot per chunk; a W8A8 unit restarts in the next slot at each fold boundary
-      // (every chunk_stages(len) stages) unless its row tile passed the exactness bound, which is
-      // first needed at the first boundary, when the scan has long finished.
-      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
-        const int ulo = kb_lo(u), uhi = kb_hi(u), per = kInt8 ? chunk_stages(uhi - ulo) : uhi - ulo;
-        int slot = q % NSLOT, kb0 = ulo, next_fold = ulo + per;
-        if (q >= NSLOT &&  // the epilogue has drained this slot's previous chunk
-            !mbar_wait_bounded(acce0 + 8 * slot, (uint32_t)(((q / NSLOT) - 1) & 1), kWaitBudgetCycles)) {
+    constexpr uint32_t idesc = idesc_f16(kMode == kModeBf16 ? 1u : 0u, BN, kBM);
+    const uint64_t ad0 = sdesc_swz(sA), bd0 = sdesc_swz(sB);
+    bool ok = true, known = false;  // known: the epilogue's exactness scan has been read
+    uint32_t fail = 0u, ph = 0u;
+    int s = 0, q = 0;  // the next stage's slot, accumulator chunks produced
+    // One accumulator slot per chunk; a W8A8 unit restarts in the next slot at each fold boundary
+    // (every chunk_stages(len) stages) unless its row tile passed the exactness bound, which is
+    // first needed at the first boundary, when the scan has long finished.
+    for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+      const int ulo = kb_lo(u), uhi = kb_hi(u), per = kInt8 ? chunk_stages(uhi - ulo) : uhi - ulo;
+      int slot = q % NSLOT, kb0 = ulo, next_fold = ulo + per;
+      if (q >= NSLOT &&  // the epilogue has drained this slot's previous chunk
+          !mbar_wait_warp(acce0 + 8 * slot, (uint32_t)(((q / NSLOT) - 1) & 1), kWaitBudgetCycles)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      uint32_t d = tmem + (uint32_t)(slot * SC);
+      for (int kb = ulo; kb < uhi; ++kb) {
+        if (kInt8 && kb == next_fold) {  // a fold boundary
+          next_fold += per;
+          if (scan && !known) {
+            if (!mbar_wait_warp(ready, 0u, kWaitBudgetCycles)) {
+              ok = false;
+              break;
+            }
+            fail = s_fail;
+            known = true;
+          }
+          if (!(scan && row_tile_exact(fail, ord.row(u / KS)))) {
+            if (elect_one()) tc_commit(accf0 + 8 * slot);
+            ++q;
+            slot = q % NSLOT;
+            if (q >= NSLOT &&
+                !mbar_wait_warp(acce0 + 8 * slot, (uint32_t)(((q / NSLOT) - 1) & 1), kWaitBudgetCycles)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            d = tmem + (uint32_t)(slot * SC);
+            kb0 = kb;
+          }
+        }
+        if (!mbar_wait_warp(full0 + 8 * s, ph, kWaitBudgetCycles)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        uint32_t d = tmem + (uint32_t)(slot * SC);
-        for (int kb = ulo; kb < uhi; ++kb, ++g) {
-          if (kInt8 && kb == next_fold) {  // a fold boundary
-            next_fold += per;
-            if (scan && !known) {
-              if (!mbar_wait_bounded(ready, 0u, kWaitBudgetCycles)) {
-                ok = false;
-                break;
-              }
-              fail = s_fail;
-              known = true;
-            }
-            if (!(scan && row_tile_exact(fail, ord.row(u / KS)))) {
-              tc_commit(accf0 + 8 * slot);
-              ++q;
-              slot = q % NSLOT;
-              if (q >= NSLOT &&
-                  !mbar_wait_bounded(acce0 + 8 * slot, (uint32_t)(((q / NSLOT) - 1) & 1), kWaitBudgetCycles)) {
-                ok = false;
-                break;
-              }
-              tc_fence_after();
-              d = tmem + (uint32_t)(slot * SC);
-              kb0 = kb;
-            }
-          }
-          const int s = g % S;
-          if (!mbar_wait_bounded(full0 + 8 * s, (uint32_t)((g / S) & 1), kWaitBudgetCycles)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
+        const uint64_t ad = ad0 + (uint32_t)(s * (int)(kABytes >> 4)), bd = bd0 + (uint32_t)(s * (int)(GG::BBytes >> 4));
+        if (elect_one()) {
 #pragma unroll
-          for (int k16 = 0; k16 < kSwz / 32; ++k16) {  // 32 bytes of k per instruction
-            const uint64_t ad = sdesc_swz(sA + (uint32_t)s * kABytes + 32u * k16);
-            const uint64_t bd = sdesc_swz(sB + (uint32_t)s * GG::BBytes + 32u * k16);
-            tc_mma_m<kMode>(d, ad, bd, idesc, (kb == kb0 && k16 == 0) ? 0u : 1u);
-          }
+          for (int k16 = 0; k16 < kSwz / 32; ++k16)  // 32 bytes of k per instruction
+            tc_mma_m<kMode>(d, ad + 2 * k16, bd + 2 * k16, idesc, k16 > 0 || kb != kb0);
           tc_commit(empty0 + 8 * s);
         }
-        if (ok) tc_commit(accf0 + 8 * slot);
-        ++q;
+        __syncwarp();
+        if (++s == S) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
+      if (ok && elect_one()) tc_commit(accf0 + 8 * slot);
+      ++q;
+    }
+    if (elect_one()) {
       if (!ok) atomicOr(a.err, DEVERR_PRODUCER_WAIT);
       tc_commit(done);  // completes once every MMA issued above has completed
       if (!mbar_wait_bounded(done, 0u, kWaitBudgetCycles)) atomicOr(a.err, DEVERR_DRAIN_WAIT);
     }
+    __syncwarp();
   } else {
     // ---------------------------------------------------------------------- epilogue warps 0-15
     if (scan) scan_exact(a, kBM, &s_fail, ready);
@@ -503,6 +607,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t lane_base = tmem + ((uint32_t)(32 * quad) << 16);
     const bool want_top = a.kind == EPI_F32 && a.top1 != nullptr;
     const uint32_t buf = stg + (uint32_t)(warp * kStageBufBytes);
+    const f32x2 nz = f2_neg_zero();
     bool ok = true;
     int q = 0;
     // split-K partials (bf16 outputs only): unit u's block of R rows x BN columns, row-major; a
@@ -516,13 +621,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int k = 0; k < 8; ++k)
         __stcg(reinterpret_cast<uint4*>(p) + k, make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]));
     };
+    constexpr int NG = tile_groups(BN);  // this warp's 32-column groups: part NG + i
     for (int u = blockIdx.x; u < units; u += gridDim.x) {
       const int t = u / KS, n0 = ord.col(t) * BN, m0 = ord.row(t) * kBM;
       const int row = m0 + rloc;
-      unsigned long long best = 0ull;
-      auto emit32 = [&](int c0, const float (&v)[32]) {
-        stage_cols32(a, &tmY, buf, m0 + 32 * quad, n0 + c0, lane, v, want_top, best);
-      };
       // After this unit's partials are stored: true when the unit is the tile's last to arrive (it
       // then sums all parts in part order); false, or a failed wait anywhere in the epilogue, ends it.
       auto arrive_last = [&]() -> bool {
@@ -541,137 +643,90 @@ __global__ void __launch_bounds__(kThreads, 1)
         __threadfence();
         return true;
       };
+      auto wait_slot = [&](int slot) {
+        if (!mbar_wait_bounded(accf0 + 8 * slot, (uint32_t)((q / NSLOT) & 1), kWaitBudgetCycles)) {
+          ok = false;
+          atomicOr(a.err, DEVERR_CONSUMER_WAIT);
+          return false;
+        }
+        tc_fence_after();
+        return true;
+      };
+      // column values, row scale and the row's best key: loaded before the first wait, so that they
+      // overlap the MMAs
+      ColVals<NG> cv;
+      if (KS == 1) load_colvals<NG>(a, kMode != kModeBf16, n0, part, BN, lane, cv);
+      const float sx = kMode != kModeBf16 && KS == 1 && row < a.M ? a.s_x[row] : 0.0f;
+      Top top{key_value(want_top && row < a.M ? __ldcg(a.top_keys + row) : 0ull), 0ull};
+      int sums[kInt8 ? 32 * NG : 1];
+      bool folded = false;
       if constexpr (kInt8) {
-        constexpr int NG = (BN / 32 + kParts - 1) / kParts;  // this warp's 32-column groups: part + kParts i
-        int isum[32 * NG];
-#pragma unroll
-        for (int j = 0; j < 32 * NG; ++j) isum[j] = 0;
         const int nch = unit_chunks(u);
-        ColVals<NG> cv;  // before the first wait: the loads overlap the MMAs
-        if (KS == 1) load_colvals<NG>(a, true, n0, part, BN, lane, cv);
-        const float sx = KS == 1 && row < a.M ? a.s_x[row] : 0.0f;
-        if (nch == 1 && KS == 1) {  // one exact fp32 accumulator: the INT32 sum as a float
-          const int slot = q % NSLOT;
-          if (!mbar_wait_bounded(accf0 + 8 * slot, (uint32_t)((q / NSLOT) & 1), kWaitBudgetCycles)) {
-            ok = false;
-            atomicOr(a.err, DEVERR_CONSUMER_WAIT);
-            break;
-          }
-          tc_fence_after();
+        folded = nch > 1 || KS > 1;
+        if (folded) {
+          int isum[32 * NG];
 #pragma unroll
-          for (int i = 0; i < NG; ++i) {
-            const int g = part + kParts * i;
-            if (g >= BN / 32) break;
-            uint32_t r[32];
-            tmem_ld32(lane_base + (uint32_t)(slot * SC + 32 * g), r);
-            if (a.acc_dbg && row < a.M) {
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (n0 + 32 * g + j < a.N)
-                  a.acc_dbg[(size_t)row * a.N + n0 + 32 * g + j] = __float2int_rn(__uint_as_float(r[j]));
-            }
-            float v[32];
-            dequant32(a.bias != nullptr, sx, cv.sw[i], cv.b[i], r, v);
-            emit32(32 * g, v);
-          }
-          tc_fence_before();
-          mbar_arrive(acce0 + 8 * slot);
-          ++q;
-          if (want_top && row < a.M && best != 0ull) atomicMax(a.top_keys + row, best);
-          continue;
-        }
-        for (int c = 0; c < nch; ++c, ++q) {
-          const int slot = q % NSLOT;
-          if (!mbar_wait_bounded(accf0 + 8 * slot, (uint32_t)((q / NSLOT) & 1), kWaitBudgetCycles)) {
-            ok = false;
-            atomicOr(a.err, DEVERR_CONSUMER_WAIT);
-            break;
-          }
-          tc_fence_after();
-#pragma unroll
-          for (int i = 0; i < NG; ++i) {
-            const int g = part + kParts * i;
-            if (g >= BN / 32) break;
-            uint32_t r[32];
-            tmem_ld32(lane_base + (uint32_t)(slot * SC + 32 * g), r);
-#pragma unroll
-            for (int j = 0; j < 32; ++j) isum[32 * i + j] += __float2int_rn(__uint_as_float(r[j]));
-          }
-          tc_fence_before();
-          mbar_arrive(acce0 + 8 * slot);
-        }
-        if (KS > 1) {
-          if (ok && has_row) {
+          for (int j = 0; j < 32 * NG; ++j) isum[j] = 0;
+          for (int c = 0; c < nch; ++c, ++q) {
+            const int slot = q % NSLOT;
+            if (!wait_slot(slot)) break;
 #pragma unroll
             for (int i = 0; i < NG; ++i) {
-              const int g = part + kParts * i;
+              const int g = NG * part + i;
+              if (g >= BN / 32) break;
+              uint32_t r[32];
+              tmem_ld32(lane_base + (uint32_t)(slot * SC + 32 * g), r);
+#pragma unroll
+              for (int j = 0; j < 32; ++j) isum[32 * i + j] += __float2int_rn(__uint_as_float(r[j]));
+            }
+            tc_fence_before();
+            mbar_arrive(acce0 + 8 * slot);
+          }
+          if (KS > 1 && ok && has_row) {
+#pragma unroll
+            for (int i = 0; i < NG; ++i) {
+              const int g = NG * part + i;
               if (g >= BN / 32) break;
               store_part32(u, g, reinterpret_cast<const uint32_t(&)[32]>(isum[32 * i]));
             }
           }
-          if (arrive_last()) split_reduce<kModeI8, BN>(a, t * KS, KS, R, m0, n0);
-          if (!ok) break;
-          continue;
-        } else if (!ok) {
-          break;
-        }
 #pragma unroll
-        for (int i = 0; i < NG; ++i) {
-          const int g = part + kParts * i;
-          if (g >= BN / 32) break;
-          if (a.acc_dbg && row < a.M) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (n0 + 32 * g + j < a.N) a.acc_dbg[(size_t)row * a.N + n0 + 32 * g + j] = isum[32 * i + j];
-          }
-          float v[32];
-          dequant32(a.bias != nullptr, sx, cv.sw[i], cv.b[i], &isum[32 * i], v);
-          emit32(32 * g, v);
+          for (int j = 0; j < 32 * NG; ++j) sums[j] = isum[j];
         }
-      } else {
-        constexpr int NG = (BN / 32 + kParts - 1) / kParts;
-        ColVals<NG> cv;  // before the wait: the loads overlap the MMAs
-        if (KS == 1) load_colvals<NG>(a, kFp8, n0, part, BN, lane, cv);
-        const float sx = kFp8 && KS == 1 && row < a.M ? a.s_x[row] : 0.0f;
+      } else if (KS > 1) {  // this part's fp32 sums go to the partials
         const int slot = q % NSLOT;
-        if (!mbar_wait_bounded(accf0 + 8 * slot, (uint32_t)((q / NSLOT) & 1), kWaitBudgetCycles)) {
-          ok = false;
-          atomicOr(a.err, DEVERR_CONSUMER_WAIT);
-        } else {
-          tc_fence_after();
+        if (wait_slot(slot)) {
 #pragma unroll
           for (int i = 0; i < NG; ++i) {
-            const int g = part + kParts * i;
+            const int g = NG * part + i;
             if (g >= BN / 32) break;
             uint32_t r[32];
             tmem_ld32(lane_base + (uint32_t)(slot * SC + 32 * g), r);
-            if (KS > 1) {  // this part's fp32 sums go to the partials
-              if (has_row) store_part32(u, g, r);
-              continue;
-            }
-            float v[32];
-            if constexpr (kFp8) {
-              dequant32(a.bias != nullptr, sx, cv.sw[i], cv.b[i], r, v);
-            } else {
-#pragma unroll
-              for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-              if (a.bias) add_bias32(cv.b[i], v);
-            }
-            emit32(32 * g, v);
+            if (has_row) store_part32(u, g, r);
           }
           tc_fence_before();
           mbar_arrive(acce0 + 8 * slot);
         }
         ++q;
-        if (KS > 1) {
-          if (arrive_last()) split_reduce<kMode, BN>(a, t * KS, KS, R, m0, n0);
-          if (!ok) break;
-          continue;
-        } else if (!ok) {
-          break;
-        }
       }
-      if (want_top && row < a.M && best != 0ull) atomicMax(a.top_keys + row, best);
+      if (KS > 1) {
+        if (arrive_last()) split_reduce<kMode, BN>(a, t * KS, KS, R, m0, n0);
+        if (!ok) break;
+        continue;
+      }
+      const int slot = q % NSLOT;
+      if (!folded) {
+        if (!wait_slot(slot)) break;
+        ++q;
+      } else if (!ok) {
+        break;
+      }
+      emit_tile<kMode, BN, NG>(a, &tmY, buf, folded, sums, lane_base + (uint32_t)(slot * SC), m0 + 32 * quad, n0, part,
+                               lane, cv, sx, want_top, nz, top, [&] {
+                                 tc_fence_before();
+                                 mbar_arrive(acce0 + 8 * slot);
+                               });
+      if (want_top && row < a.M && top.best != 0ull) atomicMax(a.top_keys + row, top.best);
     }
     if (lane == 0) bulk_wait_all();  // this warp's output stores have completed
     __syncwarp();
@@ -851,22 +906,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 
   if (warp == kProdWarp) {
     // ---------------------------------------------------------------------- TMA producers (both CTAs)
-    if (lane == 0) {
-      bool ok = true;
-      int g = 0;
-      for (int t = pair; t < tiles && ok; t += npairs) {
-        const int n0 = ord.col(t) * BN, m0 = ord.row(t) * 2 * kBM;
-        for (int kb = 0; kb < nkb; ++kb, ++g) {
-          const int s = g % S;
-          if (!mbar_wait_bounded(empty0 + 8 * s, (uint32_t)(((g / S) & 1) ^ 1), kWaitBudgetCycles)) {
-            ok = false;
-            break;
-          }
+    bool ok = true;
+    int g = 0, s = 0;
+    uint32_t ph = 1;
+    for (int t = pair; t < tiles && ok; t += npairs) {
+      const int n0 = ord.col(t) * BN + (BN / 2) * (int)rank, m0 = ord.row(t) * 2 * kBM + kBM * (int)rank;
+      for (int kb = 0; kb < nkb; ++kb, ++g) {
+        if (!mbar_wait_warp(empty0 + 8 * s, ph, kWaitBudgetCycles)) {
+          ok = false;
+          break;
+        }
+        if (elect_one()) {
           if (rank == 0) mbar_arrive_expect_tx(full0 + 8 * s, 2 * (kABytes + GG::BHalf));
-          tma_load_2d_pair(sA + (uint32_t)s * kABytes, &tmA, kb * BKe, m0 + kBM * (int)rank, full_lead + 8 * s);
-          tma_load_2d_pair(sB + (uint32_t)s * GG::BHalf, &tmB, kb * BKe, n0 + (BN / 2) * (int)rank, full_lead + 8 * s);
+          tma_load_2d_pair(sA + (uint32_t)s * kABytes, &tmA, kb * BKe, m0, full_lead + 8 * s);
+          tma_load_2d_pair(sB + (uint32_t)s * GG::BHalf, &tmB, kb * BKe, n0, full_lead + 8 * s);
+        }
+        __syncwarp();
+        if (++s == S) {
+          s = 0;
+          ph ^= 1u;
         }
       }
+    }
+    if (lane == 0) {
       if (!ok) atomicOr(a.err, DEVERR_PRODUCER_WAIT);
       // the last stages are consumed (so their copies have landed) before this CTA can exit
       for (int j = g > S ? g - S : 0; j < g; ++j) {
@@ -878,27 +940,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
   } else if (warp == kMmaWarp) {
     // ---------------------------------------------------------------------- MMA issuer (CTA 0)
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       constexpr uint32_t idesc = idesc_f16(kMode == kModeBf16 ? 1u : 0u, BN, 2 * kBM);
+      const uint64_t ad0 = sdesc_swz(sA), bd0 = sdesc_swz(sB);
       bool ok = true, known = false;  // known: this CTA's exactness scan has been read
-      uint32_t fail = 0u;
-      int g = 0, q = 0;
+      uint32_t fail = 0u, ph = 0u;
+      int s = 0, q = 0;
       // As in the single-CTA kernel: a W8A8 tile restarts in the next slot at each fold boundary
       // unless its row tile passed the exactness bound.
       for (int t = pair; t < tiles && ok; t += npairs) {
         int slot = q % NSLOT, kb0 = 0, next_fold = kb_per_chunk;
         if (q >= NSLOT &&
-            !mbar_wait_bounded(acce0 + 8 * slot, (uint32_t)(((q / NSLOT) - 1) & 1), kWaitBudgetCycles)) {
+            !mbar_wait_warp(acce0 + 8 * slot, (uint32_t)(((q / NSLOT) - 1) & 1), kWaitBudgetCycles)) {
           ok = false;
           break;
         }
         tc_fence_after();
         uint32_t d = tmem + (uint32_t)(slot * SC);
-        for (int kb = 0; kb < nkb; ++kb, ++g) {
+        for (int kb = 0; kb < nkb; ++kb) {
           if (kInt8 && kb == next_fold) {  // a fold boundary
             next_fold += kb_per_chunk;
             if (scan && !known) {
-              if (!mbar_wait_bounded(ready, 0u, kWaitBudgetCycles)) {
+              if (!mbar_wait_warp(ready, 0u, kWaitBudgetCycles)) {
                 ok = false;
                 break;
               }
@@ -906,11 +969,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
               known = true;
             }
             if (!(scan && row_tile_exact(fail, ord.row(t)))) {
-              tc2_commit_both(accf0 + 8 * slot);
+              if (elect_one()) tc2_commit_both(accf0 + 8 * slot);
               ++q;
               slot = q % NSLOT;
               if (q >= NSLOT &&
-                  !mbar_wait_bounded(acce0 + 8 * slot, (uint32_t)(((q / NSLOT) - 1) & 1), kWaitBudgetCycles)) {
+                  !mbar_wait_warp(acce0 + 8 * slot, (uint32_t)(((q / NSLOT) - 1) & 1), kWaitBudgetCycles)) {
                 ok = false;
                 break;
               }
@@ -919,26 +982,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
               kb0 = kb;
             }
           }
-          const int s = g % S;
-          if (!mbar_wait_bounded(full0 + 8 * s, (uint32_t)((g / S) & 1), kWaitBudgetCycles)) {
+          if (!mbar_wait_warp(full0 + 8 * s, ph, kWaitBudgetCycles)) {
             ok = false;
             break;
           }
           tc_fence_after();
+          const uint64_t ad = ad0 + (uint32_t)(s * (int)(kABytes >> 4)), bd = bd0 + (uint32_t)(s * (int)(GG::BHalf >> 4));
+          if (elect_one()) {
 #pragma unroll
-          for (int k16 = 0; k16 < kSwz / 32; ++k16) {  // 32 bytes of k per instruction
-            const uint64_t ad = sdesc_swz(sA + (uint32_t)s * kABytes + 32u * k16);
-            const uint64_t bd = sdesc_swz(sB + (uint32_t)s * GG::BHalf + 32u * k16);
-            tc2_mma_m<kMode>(d, ad, bd, idesc, (kb == kb0 && k16 == 0) ? 0u : 1u);
+            for (int k16 = 0; k16 < kSwz / 32; ++k16)  // 32 bytes of k per instruction
+              tc2_mma_m<kMode>(d, ad + 2 * k16, bd + 2 * k16, idesc, k16 > 0 || kb != kb0);
+            tc2_commit_both(empty0 + 8 * s);
           }
-          tc2_commit_both(empty0 + 8 * s);
+          __syncwarp();
+          if (++s == S) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
-        if (ok) tc2_commit_both(accf0 + 8 * slot);
+        if (ok && elect_one()) tc2_commit_both(accf0 + 8 * slot);
         ++q;
       }
-      if (!ok) atomicOr(a.err, DEVERR_PRODUCER_WAIT);
-      tc2_commit(done);
-      if (!mbar_wait_bounded(done, 0u, kWaitBudgetCycles)) atomicOr(a.err, DEVERR_DRAIN_WAIT);
+      if (elect_one()) {
+        if (!ok) atomicOr(a.err, DEVERR_PRODUCER_WAIT);
+        tc2_commit(done);
+        if (!mbar_wait_bounded(done, 0u, kWaitBudgetCycles)) atomicOr(a.err, DEVERR_DRAIN_WAIT);
+      }
+      __syncwarp();
     }
   } else {
     // ---------------------------------------------------------------------- epilogue warps 0-15 (both CTAs)
@@ -947,121 +1017,67 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const uint32_t lane_base = tmem + ((uint32_t)(32 * quad) << 16);
     const bool want_top = a.kind == EPI_F32 && a.top1 != nullptr;
     const uint32_t buf = stg + (uint32_t)(warp * kStageBufBytes);
+    const f32x2 nz = f2_neg_zero();
+    constexpr int NG = tile_groups(BN);  // this warp's 32-column groups: part NG + i
     bool ok = true;
     int q = 0;
-    for (int t = pair; t < tiles && ok; t += npairs) {
+    for (int t = pair; t < tiles; t += npairs) {
       const int n0 = ord.col(t) * BN, m0 = ord.row(t) * 2 * kBM;
       const int row = m0 + kBM * (int)rank + 32 * quad + lane;
-      unsigned long long best = 0ull;
-      auto emit = [&](int c0, const float (&v)[32]) {
-        stage_cols32(a, &tmY, buf, m0 + kBM * (int)rank + 32 * quad, n0 + c0, lane, v, want_top, best);
-      };
-      if constexpr (kInt8) {
-        constexpr int NG = (BN / 32 + kParts - 1) / kParts;  // this warp's 32-column groups: part + kParts i
-        int isum[32 * NG];
-#pragma unroll
-        for (int j = 0; j < 32 * NG; ++j) isum[j] = 0;
-        ColVals<NG> cv;  // before the first wait: the loads overlap the MMAs
-        load_colvals<NG>(a, true, n0, part, BN, lane, cv);
-        const float sx = row < a.M ? a.s_x[row] : 0.0f;
-        const int nch = tile_chunks(t);
-        if (nch == 1) {  // one exact fp32 accumulator: it is the INT32 sum as a float; dequantise directly
-          const int slot = q % NSLOT;
-          if (!mbar_wait_bounded(accf0 + 8 * slot, (uint32_t)((q / NSLOT) & 1), kWaitBudgetCycles)) {
-            ok = false;
-            atomicOr(a.err, DEVERR_CONSUMER_WAIT);
-            break;
-          }
-          tc_fence_after();
-#pragma unroll
-          for (int i = 0; i < NG; ++i) {
-            const int g = part + kParts * i;
-            if (g >= BN / 32) break;
-            uint32_t r[32];
-            tmem_ld32(lane_base + (uint32_t)(slot * SC + 32 * g), r);
-            if (a.acc_dbg && row < a.M) {
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (n0 + 32 * g + j < a.N)
-                  a.acc_dbg[(size_t)row * a.N + n0 + 32 * g + j] = __float2int_rn(__uint_as_float(r[j]));
-            }
-            float v[32];
-            dequant32(a.bias != nullptr, sx, cv.sw[i], cv.b[i], r, v);
-            emit(32 * g, v);
-          }
-          tc_fence_before();
-          mbar_arrive_cluster(acce_lead + 8 * slot);
-          ++q;
-          if (want_top && row < a.M && best != 0ull) atomicMax(a.top_keys + row, best);
-          continue;
-        }
-        for (int c = 0; c < nch; ++c, ++q) {
-          const int slot = q % NSLOT;
-          if (!mbar_wait_bounded(accf0 + 8 * slot, (uint32_t)((q / NSLOT) & 1), kWaitBudgetCycles)) {
-            ok = false;
-            atomicOr(a.err, DEVERR_CONSUMER_WAIT);
-            break;
-          }
-          tc_fence_after();
-#pragma unroll
-          for (int i = 0; i < NG; ++i) {
-            const int g = part + kParts * i;
-            if (g >= BN / 32) break;
-            uint32_t r[32];
-            tmem_ld32(lane_base + (uint32_t)(slot * SC + 32 * g), r);
-#pragma unroll
-            for (int j = 0; j < 32; ++j) isum[32 * i + j] += __float2int_rn(__uint_as_float(r[j]));
-          }
-          tc_fence_before();
-          mbar_arrive_cluster(acce_lead + 8 * slot);
-        }
-        if (!ok) break;
-#pragma unroll
-        for (int i = 0; i < NG; ++i) {
-          const int g = part + kParts * i;
-          if (g >= BN / 32) break;
-          if (a.acc_dbg && row < a.M) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (n0 + 32 * g + j < a.N) a.acc_dbg[(size_t)row * a.N + n0 + 32 * g + j] = isum[32 * i + j];
-          }
-          float v[32];
-          dequant32(a.bias != nullptr, sx, cv.sw[i], cv.b[i], &isum[32 * i], v);
-          emit(32 * g, v);
-        }
-      } else {
-        constexpr int NG = (BN / 32 + kParts - 1) / kParts;
-        ColVals<NG> cv;  // before the wait: the loads overlap the MMAs
-        load_colvals<NG>(a, kFp8, n0, part, BN, lane, cv);
-        const float sx = kFp8 && row < a.M ? a.s_x[row] : 0.0f;
-        const int slot = q % NSLOT;
+      auto wait_slot = [&](int slot) {
         if (!mbar_wait_bounded(accf0 + 8 * slot, (uint32_t)((q / NSLOT) & 1), kWaitBudgetCycles)) {
           ok = false;
           atomicOr(a.err, DEVERR_CONSUMER_WAIT);
-          break;
+          return false;
         }
         tc_fence_after();
+        return true;
+      };
+      ColVals<NG> cv;  // loaded before the first wait, like the row's scale and best key: the loads overlap the MMAs
+      load_colvals<NG>(a, kMode != kModeBf16, n0, part, BN, lane, cv);
+      const float sx = kMode != kModeBf16 && row < a.M ? a.s_x[row] : 0.0f;
+      Top top{key_value(want_top && row < a.M ? __ldcg(a.top_keys + row) : 0ull), 0ull};
+      int sums[kInt8 ? 32 * NG : 1];
+      bool folded = false;
+      if constexpr (kInt8) {
+        const int nch = tile_chunks(t);
+        folded = nch > 1;
+        if (folded) {
+          int isum[32 * NG];
 #pragma unroll
-        for (int i = 0; i < NG; ++i) {
-          const int g = part + kParts * i;
-          if (g >= BN / 32) break;
-          uint32_t r[32];
-          tmem_ld32(lane_base + (uint32_t)(slot * SC + 32 * g), r);
-          float v[32];
-          if constexpr (kFp8) {
-            dequant32(a.bias != nullptr, sx, cv.sw[i], cv.b[i], r, v);
-          } else {
+          for (int j = 0; j < 32 * NG; ++j) isum[j] = 0;
+          for (int c = 0; c < nch; ++c, ++q) {
+            const int slot = q % NSLOT;
+            if (!wait_slot(slot)) break;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-            if (a.bias) add_bias32(cv.b[i], v);
+            for (int i = 0; i < NG; ++i) {
+              const int g = NG * part + i;
+              if (g >= BN / 32) break;
+              uint32_t r[32];
+              tmem_ld32(lane_base + (uint32_t)(slot * SC + 32 * g), r);
+#pragma unroll
+              for (int j = 0; j < 32; ++j) isum[32 * i + j] += __float2int_rn(__uint_as_float(r[j]));
+            }
+            tc_fence_before();
+            mbar_arrive_cluster(acce_lead + 8 * slot);
           }
-          emit(32 * g, v);
+#pragma unroll
+          for (int j = 0; j < 32 * NG; ++j) sums[j] = isum[j];
         }
-        tc_fence_before();
-        mbar_arrive_cluster(acce_lead + 8 * slot);
-        ++q;
       }
-      if (want_top && row < a.M && best != 0ull) atomicMax(a.top_keys + row, best);
+      const int slot = q % NSLOT;
+      if (!folded) {
+        if (!wait_slot(slot)) break;
+        ++q;
+      } else if (!ok) {
+        break;
+      }
+      emit_tile<kMode, BN, NG>(a, &tmY, buf, folded, sums, lane_base + (uint32_t)(slot * SC),
+                               m0 + kBM * (int)rank + 32 * quad, n0, part, lane, cv, sx, want_top, nz, top, [&] {
+                                 tc_fence_before();
+                                 mbar_arrive_cluster(acce_lead + 8 * slot);
+                               });
+      if (want_top && row < a.M && top.best != 0ull) atomicMax(a.top_keys + row, top.best);
     }
     if (lane == 0) bulk_wait_all();  // this warp's output stores have completed
     __syncwarp();
@@ -1092,13 +1108,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   }
 }
 
-// The output's tensor map for the epilogue's TMA stores: 32 rows x 32 bf16 columns, or 16 (GeGLU
-// output, fp32 logits), swizzled over the staged row's width.
-w8a8_status make_out_map(const TcArgs& a, CUtensorMap* ty, const CUtensorMap& unused) {
-  if (a.kind == EPI_BF16) return make_tmap_2d(ty, a.y, 2, (uint64_t)a.N, (uint64_t)a.M, (uint64_t)a.N * 2, 32, 32, 64);
-  if (a.kind == EPI_GEGLU)
-    return make_tmap_2d(ty, a.y, 2, (uint64_t)(a.N / 2), (uint64_t)a.M, (uint64_t)a.N, 16, 32, 32);
-  if (a.logits) return make_tmap_2d(ty, a.logits, 4, (uint64_t)a.N, (uint64_t)a.M, (uint64_t)a.N * 4, 16, 32, 64);
+// The output's tensor map for the epilogue's TMA stores: the epilogue's block (ng: 32-column groups
+// per warp and tile), swizzled over the staged row's width.
+w8a8_status make_out_map(const TcArgs& a, int ng, CUtensorMap* ty, const CUtensorMap& unused) {
+  const uint64_t N = (uint64_t)a.N, M = (uint64_t)a.M;
+  if (a.kind == EPI_BF16) return make_tmap_2d(ty, a.y, 2, N, M, N * 2, 32, 32, 64);
+  if (a.kind == EPI_GEGLU) return make_tmap_2d(ty, a.y, 2, N / 2, M, N, 16 * ng, 32, 32 * ng);
+  if (a.logits) return make_tmap_2d(ty, a.logits, 4, N, M, N * 4, 32, 16, 128);
   *ty = unused;  // top-1 only: nothing is stored
   return W8A8_OK;
 }
@@ -1119,7 +1135,7 @@ w8a8_status launch_t(const TcArgs& a, cudaStream_t st) {
                         (uint32_t)a_box_rows(a.M), kSwz));
   W8A8_TRY(make_tmap_2d(&tb, a.B, EB, (uint64_t)a.K, (uint64_t)a.N, (uint64_t)a.K * EB, BKe, GG::BN, kSwz));
   CUtensorMap ty;
-  W8A8_TRY(make_out_map(a, &ty, ta));
+  W8A8_TRY(make_out_map(a, tile_groups(GG::BN), &ty, ta));
   const long long tiles = (long long)((a.N + GG::BN - 1) / GG::BN) * ((a.M + kBM - 1) / kBM);
   const dim3 grid((unsigned)std::min<long long>(tiles * std::max(a.ksplit, 1), device_sms()));
   W8A8_CUDA(launch_pdl(gemm_tc_kernel<kMode, kBN>, grid, dim3(kThreads), (size_t)GG::Smem, st, ta, tb, ty, a));
@@ -1141,7 +1157,7 @@ w8a8_status launch_t2(const TcArgs& a, cudaStream_t st) {
   W8A8_TRY(make_tmap_2d(&ta, a.A, EB, (uint64_t)a.K, (uint64_t)a.M, (uint64_t)a.K * EB, BKe, kBM, kSwz));
   W8A8_TRY(make_tmap_2d(&tb, a.B, EB, (uint64_t)a.K, (uint64_t)a.N, (uint64_t)a.K * EB, BKe, GG::BN / 2, kSwz));
   CUtensorMap ty;
-  W8A8_TRY(make_out_map(a, &ty, ta));
+  W8A8_TRY(make_out_map(a, tile_groups(GG::BN), &ty, ta));
   const long long tiles = (long long)((a.N + GG::BN - 1) / GG::BN) * ((a.M + 2 * kBM - 1) / (2 * kBM));
   const long long pairs = std::min<long long>(tiles, device_sms() / 2);
   W8A8_CUDA(launch_pdl(gemm_tc2_kernel<kMode, kBN>, dim3((unsigned)(2 * pairs)), dim3(kThreads), (size_t)GG::Smem, st,
