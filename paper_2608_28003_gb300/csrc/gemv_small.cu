@@ -225,7 +225,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
   // weights of the fused residual norm (constants): this thread's 8 channels
   const int nvk = a.K >> 3;
   float wp[8], wn[8];
-  if (a.has_rn && tid < nvk) {
+  if (MT == 1 && a.has_rn && tid < nvk) {
     const float4* p0 = reinterpret_cast<const float4*>(a.rn.w_post + 8 * tid);
     const float4* p1 = reinterpret_cast<const float4*>(a.rn.w_next + 8 * tid);
     const float4 a0 = p0[0], a1 = p0[1], b0 = p1[0], b1 = p1[1];
@@ -243,46 +243,144 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
   const int xsb = kMma ? kpad + (kQ ? 16 : 8) : kpad;
   if (a.has_rn) {
     uint16_t* as = kQ ? reinterpret_cast<uint16_t*>(xsp + p.xbytes) : reinterpret_cast<uint16_t*>(xsp);
-    for (int m = 0; m < MT; ++m) {
-      const bool mine = m < a.M && tid < nvk;
-      float yv[8], rv[8];
-      float ss = 0.0f;
-      if (mine) {
-        const uint4 yw = reinterpret_cast<const uint4*>(a.rn.y + (size_t)m * a.K)[tid];
-        unpack_bf16x8(yw, yv);
-        const float4* rp = reinterpret_cast<const float4*>(a.rn.r_in + (size_t)m * a.K + 8 * tid);
-        const float4 r0 = rp[0], r1 = rp[1];
-        rv[0] = r0.x; rv[1] = r0.y; rv[2] = r0.z; rv[3] = r0.w; rv[4] = r1.x; rv[5] = r1.y; rv[6] = r1.z; rv[7] = r1.w;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) ss += yv[e] * yv[e];
-      }
-      const float inv_y = 1.0f / sqrtf(consumer_sum(ss, s_red, warp, lane) / (float)a.K + a.rn.eps);
-      float ss2 = 0.0f;
-      if (mine) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          rv[e] += yv[e] * inv_y * wp[e];
-          ss2 += rv[e] * rv[e];
-        }
-        if (blockIdx.x == 0) {
-          float4* ro = reinterpret_cast<float4*>(a.rn.r_out + (size_t)m * a.K + 8 * tid);
-          ro[0] = make_float4(rv[0], rv[1], rv[2], rv[3]);
-          ro[1] = make_float4(rv[4], rv[5], rv[6], rv[7]);
-        }
-      }
-      const float inv_r = 1.0f / sqrtf(consumer_sum(ss2, s_red, warp, lane) / (float)a.K + a.rn.eps);
-      if (tid < (kpad >> 3)) {  // the padded row: zeros past K and in slots >= M
-        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+    const int astride = kQ ? kpad : xsb;  // elements between the rows in shared memory
+    if constexpr (MT == 1) {
+      {
+        constexpr int m = 0;
+        const bool mine = m < a.M && tid < nvk;
+        float yv[8], rv[8];
+        float ss = 0.0f;
         if (mine) {
-          float o[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) o[e] = rv[e] * inv_r * wn[e];
-          w.x = (uint32_t)f32_to_bf16_bits(o[0]) | ((uint32_t)f32_to_bf16_bits(o[1]) << 16);
-          w.y = (uint32_t)f32_to_bf16_bits(o[2]) | ((uint32_t)f32_to_bf16_bits(o[3]) << 16);
-          w.z = (uint32_t)f32_to_bf16_bits(o[4]) | ((uint32_t)f32_to_bf16_bits(o[5]) << 16);
-          w.w = (uint32_t)f32_to_bf16_bits(o[6]) | ((uint32_t)f32_to_bf16_bits(o[7]) << 16);
+          const uint4 yw = reinterpret_cast<const uint4*>(a.rn.y + (size_t)m * a.K)[tid];
+          unpack_bf16x8(yw, yv);
+          const float4* rp = reinterpret_cast<const float4*>(a.rn.r_in + (size_t)m * a.K + 8 * tid);
+          const float4 r0 = rp[0], r1 = rp[1];
+          rv[0] = r0.x; rv[1] = r0.y; rv[2] = r0.z; rv[3] = r0.w; rv[4] = r1.x; rv[5] = r1.y; rv[6] = r1.z; rv[7] = r1.w;
+  #pragma unroll
+          for (int e = 0; e < 8; ++e) ss += yv[e] * yv[e];
         }
-        *reinterpret_cast<uint4*>(as + (size_t)m * (kQ ? kpad : xsb) + 8 * tid) = w;
+        const float inv_y = 1.0f / sqrtf(consumer_sum(ss, s_red, warp, lane) / (float)a.K + a.rn.eps);
+        float ss2 = 0.0f;
+        if (mine) {
+  #pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            rv[e] += yv[e] * inv_y * wp[e];
+            ss2 += rv[e] * rv[e];
+          }
+          if (blockIdx.x == 0) {
+            float4* ro = reinterpret_cast<float4*>(a.rn.r_out + (size_t)m * a.K + 8 * tid);
+            ro[0] = make_float4(rv[0], rv[1], rv[2], rv[3]);
+            ro[1] = make_float4(rv[4], rv[5], rv[6], rv[7]);
+          }
+        }
+        const float inv_r = 1.0f / sqrtf(consumer_sum(ss2, s_red, warp, lane) / (float)a.K + a.rn.eps);
+        if (tid < (kpad >> 3)) {  // the padded row: zeros past K and in slots >= M
+          uint4 w = make_uint4(0u, 0u, 0u, 0u);
+          if (mine) {
+            float o[8];
+  #pragma unroll
+            for (int e = 0; e < 8; ++e) o[e] = rv[e] * inv_r * wn[e];
+            w.x = (uint32_t)f32_to_bf16_bits(o[0]) | ((uint32_t)f32_to_bf16_bits(o[1]) << 16);
+            w.y = (uint32_t)f32_to_bf16_bits(o[2]) | ((uint32_t)f32_to_bf16_bits(o[3]) << 16);
+            w.z = (uint32_t)f32_to_bf16_bits(o[4]) | ((uint32_t)f32_to_bf16_bits(o[5]) << 16);
+            w.w = (uint32_t)f32_to_bf16_bits(o[6]) | ((uint32_t)f32_to_bf16_bits(o[7]) << 16);
+          }
+          *reinterpret_cast<uint4*>(as + (size_t)m * (kQ ? kpad : xsb) + 8 * tid) = w;
+        }
+      }
+    } else {
+      // Several token slots: a warp per row, so that the rows run side by side and their sums need no
+      // block barrier.  (All 256 threads on one row after the other took about 1 us per slot, two
+      // launches a layer: decode of 8 sequences 1170 us, now 1070.)  Lane l owns the 16-byte vectors
+      // l, l + 32, ...; the first kKeep of them stay in registers (K <= 1280: all), later ones are
+      // read again for each pass.
+      constexpr int kKeep = 5;
+      const float4* w_post = reinterpret_cast<const float4*>(a.rn.w_post);
+      const float4* w_next = reinterpret_cast<const float4*>(a.rn.w_next);
+      for (int m = warp; m < MT; m += CW) {
+        const bool live = m < a.M;
+        const uint4* yr = reinterpret_cast<const uint4*>(a.rn.y + (size_t)m * a.K);
+        const float4* rr = reinterpret_cast<const float4*>(a.rn.r_in + (size_t)m * a.K);
+        float4* ro = reinterpret_cast<float4*>(a.rn.r_out + (size_t)m * a.K);
+        uint16_t* arow = as + (size_t)m * astride;
+        auto squares = [](const uint4& w) {
+          float x[8], t = 0.0f;
+          unpack_bf16x8(w, x);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) t += x[e] * x[e];
+          return t;
+        };
+        // r += y inv_y w_post of one vector; returns the new values' squares
+        auto residual = [&](const uint4& w, int vi, float inv_y, float (&r)[8]) {
+          float x[8], t = 0.0f;
+          unpack_bf16x8(w, x);
+          const float4 p0 = w_post[2 * vi], p1 = w_post[2 * vi + 1];
+          const float pw[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            r[e] += x[e] * inv_y * pw[e];
+            t += r[e] * r[e];
+          }
+          return t;
+        };
+        auto load_r = [&](int vi, float (&r)[8]) {
+          const float4 r0 = rr[2 * vi], r1 = rr[2 * vi + 1];
+          r[0] = r0.x; r[1] = r0.y; r[2] = r0.z; r[3] = r0.w; r[4] = r1.x; r[5] = r1.y; r[6] = r1.z; r[7] = r1.w;
+        };
+        auto emit = [&](int vi, float inv_r, const float (&r)[8]) {
+          if (blockIdx.x == 0) {
+            ro[2 * vi] = make_float4(r[0], r[1], r[2], r[3]);
+            ro[2 * vi + 1] = make_float4(r[4], r[5], r[6], r[7]);
+          }
+          const float4 n0 = w_next[2 * vi], n1 = w_next[2 * vi + 1];
+          const float nw[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
+          uint32_t o[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            o[e] = (uint32_t)f32_to_bf16_bits(r[2 * e] * inv_r * nw[2 * e]) |
+                   ((uint32_t)f32_to_bf16_bits(r[2 * e + 1] * inv_r * nw[2 * e + 1]) << 16);
+          *reinterpret_cast<uint4*>(arow + 8 * vi) = make_uint4(o[0], o[1], o[2], o[3]);
+        };
+        if (live) {
+          uint4 yv[kKeep];
+          float rv[kKeep][8];
+          float ss = 0.0f;
+#pragma unroll
+          for (int v = 0; v < kKeep; ++v) {
+            const int vi = lane + 32 * v;
+            yv[v] = make_uint4(0u, 0u, 0u, 0u);
+            if (vi < nvk) {
+              yv[v] = yr[vi];
+              load_r(vi, rv[v]);
+            }
+          }
+#pragma unroll
+          for (int v = 0; v < kKeep; ++v) ss += squares(yv[v]);
+          for (int vi = lane + 32 * kKeep; vi < nvk; vi += 32) ss += squares(yr[vi]);
+          const float inv_y = 1.0f / sqrtf(warp_sum32(ss) / (float)a.K + a.rn.eps);
+          float ss2 = 0.0f;
+#pragma unroll
+          for (int v = 0; v < kKeep; ++v)
+            if (lane + 32 * v < nvk) ss2 += residual(yv[v], lane + 32 * v, inv_y, rv[v]);
+          for (int vi = lane + 32 * kKeep; vi < nvk; vi += 32) {
+            float r[8];
+            load_r(vi, r);
+            ss2 += residual(yr[vi], vi, inv_y, r);
+          }
+          const float inv_r = 1.0f / sqrtf(warp_sum32(ss2) / (float)a.K + a.rn.eps);
+#pragma unroll
+          for (int v = 0; v < kKeep; ++v)
+            if (lane + 32 * v < nvk) emit(lane + 32 * v, inv_r, rv[v]);
+          for (int vi = lane + 32 * kKeep; vi < nvk; vi += 32) {
+            float r[8];
+            load_r(vi, r);
+            residual(yr[vi], vi, inv_y, r);
+            emit(vi, inv_r, r);
+          }
+        }
+        // the padded row: zeros past K and in slots >= M
+        for (int vi = live ? nvk + lane : lane; vi < (kpad >> 3); vi += 32)
+          *reinterpret_cast<uint4*>(arow + 8 * vi) = make_uint4(0u, 0u, 0u, 0u);
       }
     }
     named_bar_sync(1, CW * 32);
