@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libw8a8.so (argument marshalling only).
+"""Thin binding of libw8a8.so (argument marshalling only): ctypes, and for the per-layer compute
+calls the C module ``_calls`` (the same steps without the interpreter's cost).
 
 Every computation runs in the library's CUDA kernels; this module only turns torch tensors
 (device memory owned by the caller) into the pointers and descriptors of ``include/w8a8.h``,
@@ -190,6 +191,25 @@ def lib() -> ctypes.CDLL:
     return _LIB
 
 
+_CALLS = None
+
+
+def _calls():
+    """The C marshalling module, holding this library's addresses."""
+    global _CALLS
+    if _CALLS is None:
+        L = lib()
+        try:
+            from . import _calls as mod
+        except ImportError as e:
+            raise RuntimeError("paper_2608_28003_gb300/_calls.so is not built: run "
+                               "paper_2608_28003_gb300.build.build()") from e
+        mod.init({name: ctypes.cast(getattr(L, name), _vp).value for name in SIGNATURES}, _check, default_workspace,
+                 _DEFAULT_WS, Workspace)
+        _CALLS = mod
+    return _CALLS
+
+
 def _check(name: str, status: int) -> None:
     if status != 0:
         raise W8A8Error(name, status, lib().w8a8_last_error().decode())
@@ -342,24 +362,20 @@ def quantize_activations(X: torch.Tensor, inv_delta: torch.Tensor, stream=None):
 
 def linear(w: QWeight, X: torch.Tensor, bias: Optional[torch.Tensor] = None, debug: bool = False,
            out: Optional[torch.Tensor] = None, ws: Optional[Workspace] = None, stream=None):
+    if not debug:
+        return (_CALLS or _calls()).linear(w, X, bias, out, ws, stream)
     M = X.shape[0]
     Y = out if out is not None else torch.empty(M, w.n, dtype=torch.bfloat16, device=X.device)
     nbytes = _size("w8a8_linear_workspace_size", M, w.n, w.k)
     buf = (ws or default_workspace()).get(nbytes)
-    dbg = None
-    dbg_t = None
-    if debug:
-        dbg_t = (torch.empty(M, w.k, dtype=torch.int8, device=X.device),
-                 torch.empty(M, dtype=torch.float32, device=X.device),
-                 torch.empty(M, w.n, dtype=torch.int32, device=X.device))
-        dbg = DebugC(*(t.data_ptr() for t in dbg_t))
+    dbg_t = (torch.empty(M, w.k, dtype=torch.int8, device=X.device),
+             torch.empty(M, dtype=torch.float32, device=X.device),
+             torch.empty(M, w.n, dtype=torch.int32, device=X.device))
+    dbg = DebugC(*(t.data_ptr() for t in dbg_t))
     wc = w.c()
-    _check("w8a8_linear", lib().w8a8_linear(ctypes.byref(wc), _p(_bits(X)), M, _p(bias), _p(Y),
-                                            ctypes.byref(dbg) if dbg is not None else None, _p(buf),
-                                            buf.numel(), _stream(stream)))
-    if debug:
-        return Y, {"xq": dbg_t[0], "s_x": dbg_t[1], "acc": dbg_t[2]}
-    return Y
+    _check("w8a8_linear", lib().w8a8_linear(ctypes.byref(wc), _p(_bits(X)), M, _p(bias), _p(Y), ctypes.byref(dbg),
+                                            _p(buf), buf.numel(), _stream(stream)))
+    return Y, {"xq": dbg_t[0], "s_x": dbg_t[1], "acc": dbg_t[2]}
 
 
 def linear_noalloc(w: QWeight, X: torch.Tensor, bias: Optional[torch.Tensor] = None,
@@ -376,14 +392,7 @@ def linear_noalloc(w: QWeight, X: torch.Tensor, bias: Optional[torch.Tensor] = N
 
 def linear_bf16(W: torch.Tensor, X: torch.Tensor, bias: Optional[torch.Tensor] = None,
                 out: Optional[torch.Tensor] = None, ws: Optional[Workspace] = None, stream=None) -> torch.Tensor:
-    N, K = W.shape
-    M = X.shape[0]
-    Y = out if out is not None else torch.empty(M, N, dtype=torch.bfloat16, device=X.device)
-    nbytes = _size("w8a8_linear_bf16_workspace_size", M, N, K)
-    buf = (ws or default_workspace()).get(nbytes)
-    _check("w8a8_linear_bf16", lib().w8a8_linear_bf16(_p(_bits(W)), N, K, _p(_bits(X)), M, _p(bias), _p(Y), _p(buf),
-                                                      buf.numel(), _stream(stream)))
-    return Y
+    return (_CALLS or _calls()).linear_bf16(W, X, bias, out, ws, stream)
 
 
 @dataclass
@@ -405,15 +414,7 @@ class FfnWeights:
 
 def ffn_block(f: FfnWeights, precision: int, X: torch.Tensor, want_h: bool = False,
               out: Optional[torch.Tensor] = None, ws: Optional[Workspace] = None, stream=None):
-    M = X.shape[0]
-    Y = out if out is not None else torch.empty(M, f.hidden, dtype=torch.bfloat16, device=X.device)
-    h = torch.empty(M, f.inter, dtype=torch.bfloat16, device=X.device) if want_h else None
-    nbytes = _size("w8a8_ffn_workspace_size", M, f.hidden, f.inter)
-    buf = (ws or default_workspace()).get(nbytes)
-    fc = f.c()
-    _check("w8a8_ffn_block", lib().w8a8_ffn_block(ctypes.byref(fc), int(precision), _p(_bits(X)), M, _p(Y), _p(h),
-                                                  _p(buf), buf.numel(), _stream(stream)))
-    return (Y, h) if want_h else Y
+    return (_CALLS or _calls()).ffn_block(f, precision, X, want_h, out, ws, stream)
 
 
 # ------------------------------------------------------------------------ FP8 (e4m3) variant
@@ -474,15 +475,17 @@ def fp8_quantize_activations(X: torch.Tensor, inv_delta: torch.Tensor, stream=No
 
 def fp8_linear(w: Fp8Weight, X: torch.Tensor, bias: Optional[torch.Tensor] = None, debug: bool = False,
                out: Optional[torch.Tensor] = None, ws: Optional[Workspace] = None, stream=None):
+    if not debug:
+        return (_CALLS or _calls()).fp8_linear(w, X, bias, out, ws, stream)
     M = X.shape[0]
     Y = out if out is not None else torch.empty(M, w.n, dtype=torch.bfloat16, device=X.device)
     buf = (ws or default_workspace()).get(_size("w8a8_linear_workspace_size", M, w.n, w.k))
-    xq = torch.empty(M, w.k, dtype=torch.uint8, device=X.device) if debug else None
-    s_x = torch.empty(M, dtype=torch.float32, device=X.device) if debug else None
+    xq = torch.empty(M, w.k, dtype=torch.uint8, device=X.device)
+    s_x = torch.empty(M, dtype=torch.float32, device=X.device)
     wc = w.c()
     _check("w8a8_fp8_linear", lib().w8a8_fp8_linear(ctypes.byref(wc), _p(_bits(X)), M, _p(bias), _p(Y), _p(xq),
                                                     _p(s_x), _p(buf), buf.numel(), _stream(stream)))
-    return (Y, {"xq": xq, "s_x": s_x}) if debug else Y
+    return Y, {"xq": xq, "s_x": s_x}
 
 
 @dataclass
@@ -498,14 +501,7 @@ class Fp8FfnWeights:
 
 def fp8_ffn_block(f: Fp8FfnWeights, X: torch.Tensor, want_h: bool = False, out: Optional[torch.Tensor] = None,
                   ws: Optional[Workspace] = None, stream=None):
-    M = X.shape[0]
-    Y = out if out is not None else torch.empty(M, f.hidden, dtype=torch.bfloat16, device=X.device)
-    h = torch.empty(M, f.inter, dtype=torch.bfloat16, device=X.device) if want_h else None
-    buf = (ws or default_workspace()).get(_size("w8a8_ffn_workspace_size", M, f.hidden, f.inter))
-    fc = f.c()
-    _check("w8a8_fp8_ffn_block", lib().w8a8_fp8_ffn_block(ctypes.byref(fc), _p(_bits(X)), M, _p(Y), _p(h), _p(buf),
-                                                          buf.numel(), _stream(stream)))
-    return (Y, h) if want_h else Y
+    return (_CALLS or _calls()).fp8_ffn_block(f, X, want_h, out, ws, stream)
 
 
 @dataclass
@@ -524,18 +520,7 @@ class HeadWeights:
 def lm_head(hd: HeadWeights, precision: int, X: torch.Tensor, want_logits: bool = True,
             logits: Optional[torch.Tensor] = None, top1: Optional[torch.Tensor] = None,
             ws: Optional[Workspace] = None, stream=None):
-    M = X.shape[0]
-    if want_logits and logits is None:
-        logits = torch.empty(M, hd.vocab, dtype=torch.float32, device=X.device)
-    if top1 is None:
-        top1 = torch.empty(M, dtype=torch.int32, device=X.device)
-    nbytes = _size("w8a8_lm_head_workspace_size", M, hd.vocab, hd.hidden)
-    buf = (ws or default_workspace()).get(nbytes)
-    hc = hd.c()
-    _check("w8a8_lm_head", lib().w8a8_lm_head(ctypes.byref(hc), int(precision), _p(_bits(X)), M,
-                                              _p(logits) if want_logits else None, _p(top1), _p(buf), buf.numel(),
-                                              _stream(stream)))
-    return (logits if want_logits else None), top1
+    return (_CALLS or _calls()).lm_head(hd, precision, X, want_logits, logits, top1, ws, stream)
 
 
 # ------------------------------------------------------------------------------- decoder

@@ -1,7 +1,8 @@
 """Build libw8a8.so in-tree with nvcc for sm_103a (GB300).
 
 Each ``csrc/*.cu`` compiles to an object under ``_build/`` (in parallel), and the objects link
-into ``paper_2608_28003_gb300/libw8a8.so``.  A source newer than its object, or a header newer
+into ``paper_2608_28003_gb300/libw8a8.so``; ``csrc/calls.cc``, the binding's marshalling, compiles
+to the extension module ``_calls.so`` beside it.  A source newer than its object, or a header newer
 than the library, triggers a rebuild.  No fast-math: every rounding the header documents is an
 IEEE operation.
 """
@@ -12,12 +13,14 @@ import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libw8a8.so")
+CALLS = os.path.join(PKG, "_calls.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
@@ -44,8 +47,22 @@ def _compile(src: str, obj: str, verbose: bool) -> None:
         print(r.stdout, r.stderr)
 
 
+def _compile_calls(src: str) -> None:
+    cxx = shutil.which(os.environ.get("CXX", "g++")) or shutil.which("c++")
+    if cxx is None:
+        raise RuntimeError("g++ not found: it compiles the binding's calls")
+    tmp = CALLS + ".tmp"
+    cmd = [cxx, "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           "-I", sysconfig.get_paths()["include"], src, "-o", tmp]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed for {os.path.basename(src)}:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, CALLS)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every CUDA source for sm_103a and link libw8a8.so.  Returns the library path."""
+    """Compile every CUDA source for sm_103a and link libw8a8.so, and compile the binding's calls.
+    Returns the library path."""
     os.makedirs(BUILD, exist_ok=True)
     srcs = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
     hdr_mtime = max([os.path.getmtime(h) for h in _headers()] + [0.0])
@@ -56,6 +73,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
         jobs.append((s, o, stale))
     with cf.ThreadPoolExecutor(max_workers=max(1, min(len(jobs), os.cpu_count() or 4))) as ex:
         futs = [ex.submit(_compile, s, o, verbose) for s, o, stale in jobs if stale]
+        calls = os.path.join(CSRC, "calls.cc")
+        if force or not os.path.exists(CALLS) or os.path.getmtime(CALLS) < max(os.path.getmtime(calls), hdr_mtime):
+            futs.append(ex.submit(_compile_calls, calls))
         for f in futs:
             f.result()
     objs = [o for _, o, _ in jobs]
