@@ -47,11 +47,23 @@ w8a8_status launch_attn_decode(const uint16_t* qkv, const AttnShape& s, const in
                                const float* kn, float eps, const float* rope_cos, const float* rope_sin,
                                uint16_t* kcache, uint16_t* vcache, uint16_t* o, cudaStream_t st);
 
-// Prefill (T > 1): flash-attention-style attention of q (fp32, after QK-norm and RoPE) over the
-// cache on the tensor cores (fp16 operands, fp32 accumulation and softmax); o bf16 [M, n_q*hd].
+// Prefill (T > 1, positions pos0 .. pos0 + T - 1): attention on the tensor cores (fp16 operands, fp32
+// accumulation and softmax); o bf16 [M, n_q*hd].  launch_prefill_rope takes the place of launch_qk_rope:
+// QK-norm, RoPE and the cache write, and the operands of every key up to pos0 + T (scaled q, K and the
+// transposed V as fp16; zeros up to the next key multiple of 128).
+struct PrefillOperands {
+  uint16_t* q;   // [M][n_q*hd]
+  uint16_t* k;   // [B][n_kv][prefill_keys_pad(max_seq)][hd]
+  uint16_t* vt;  // [B][n_kv][hd][prefill_keys_pad(max_seq)]
+};
 bool attention_prefill_supported(const AttnShape& s);
-w8a8_status launch_attention_prefill(const float* q, const uint16_t* kcache, const uint16_t* vcache, const AttnShape& s,
-                                     const int* pos0, uint16_t* o, cudaStream_t st);
+int prefill_keys_pad(int max_seq);
+w8a8_status launch_prefill_rope(const uint16_t* qkv, const AttnShape& s, int pos0, const float* qn, const float* kn,
+                                float eps, const float* rope_cos, const float* rope_sin, uint16_t* kcache,
+                                uint16_t* vcache, const PrefillOperands& w, cudaStream_t st);
+// err: the device error word (a bounded wait that gave up)
+w8a8_status launch_attention_prefill(const PrefillOperands& w, const AttnShape& s, int pos0, uint16_t* o, int sms,
+                                     unsigned int* err, cudaStream_t st);
 
 // cos/sin tables [max_seq][hd/2] of RoPE with the given base, computed in fp64
 w8a8_status launch_rope_table(float* cos_t, float* sin_t, int max_seq, int hd, double base, cudaStream_t st);

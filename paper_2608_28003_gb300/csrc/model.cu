@@ -53,6 +53,7 @@ struct w8a8_model {
   uint16_t *a = nullptr, *qkv = nullptr, *o = nullptr, *y = nullptr, *h = nullptr;
   float* q = nullptr;
   uint16_t *kc = nullptr, *vc = nullptr;
+  uint16_t *pf_k = nullptr, *pf_vt = nullptr;  // one layer's prefill attention operands (PrefillOperands)
   float *cos_l = nullptr, *sin_l = nullptr, *cos_g = nullptr, *sin_g = nullptr;
   int* d_pos = nullptr;
   int32_t* d_tokens = nullptr;
@@ -146,9 +147,10 @@ bool fuse_residual(const w8a8_model* m, int M, bool calib) {
   return true;
 }
 
-// The decoder over M = B * T rows whose positions start at *m->d_pos (set by the caller).
-w8a8_status forward_core(w8a8_model* m, const int32_t* tokens, int B, int T, float* logits, int32_t* top1, bool calib,
-                         cudaStream_t st) {
+// The decoder over M = B * T rows whose positions start at *m->d_pos (set by the caller; T > 1: the
+// same as start_pos, which a decode step, T = 1, does not read).
+w8a8_status forward_core(w8a8_model* m, const int32_t* tokens, int B, int T, int start_pos, float* logits, int32_t* top1,
+                         bool calib, cudaStream_t st) {
   const w8a8_model_cfg& c = m->cfg;
   const int M = B * T, H = c.hidden, F = c.inter;
   const bool fuse = fuse_residual(m, M, calib);
@@ -199,12 +201,14 @@ w8a8_status forward_core(w8a8_model* m, const int32_t* tokens, int B, int T, flo
     }
     if (attn_decode_supported(s)) {
       W8A8_TRY(launch_attn_decode(m->qkv, s, m->d_pos, qn, kn, c.eps, cs, sn, kc, vc, m->o, st));
+    } else if (attention_prefill_supported(s)) {
+      const PrefillOperands w{reinterpret_cast<uint16_t*>(m->q), m->pf_k, m->pf_vt};
+      W8A8_TRY(launch_prefill_rope(m->qkv, s, start_pos, qn, kn, c.eps, cs, sn, kc, vc, w, st));
+      W8A8_TRY(launch_attention_prefill(w, s, start_pos, m->o, m->sms,
+                                        reinterpret_cast<unsigned int*>(static_cast<char*>(m->ws) + kErrWordOffset), st));
     } else {
       W8A8_TRY(launch_qk_rope(m->qkv, s, m->d_pos, qn, kn, c.eps, cs, sn, m->q, kc, vc, st));
-      if (attention_prefill_supported(s))
-        W8A8_TRY(launch_attention_prefill(m->q, kc, vc, s, m->d_pos, m->o, st));
-      else
-        W8A8_TRY(launch_attention(m->q, kc, vc, s, m->d_pos, 0, m->o, m->attn_ws, m->sms, st));
+      W8A8_TRY(launch_attention(m->q, kc, vc, s, m->d_pos, 0, m->o, m->attn_ws, m->sms, st));
     }
     if (calib) W8A8_TRY(launch_act_absmax(m->o, M, m->q_dim, m->stat_o(l), st));
     if (tr) W8A8_TRY(trace_copy(tr->attn, l, m->o, m->q_dim, 2));
@@ -410,6 +414,9 @@ extern "C" w8a8_status w8a8_model_create(const w8a8_model_cfg* cfg, const w8a8_l
   W8A8_MTRY(dalloc(m, &m->h, (size_t)Mx * F));
   W8A8_MTRY(dalloc(m, &m->kc, (size_t)c.layers * m->cache_layer_elems()));
   W8A8_MTRY(dalloc(m, &m->vc, (size_t)c.layers * m->cache_layer_elems()));
+  const size_t pf = (size_t)c.max_batch * m->kv_dim * prefill_keys_pad(c.max_seq);
+  W8A8_MTRY(dalloc(m, &m->pf_k, pf));
+  W8A8_MTRY(dalloc(m, &m->pf_vt, pf));
   const size_t rope = (size_t)c.max_seq * (c.head_dim / 2);
   W8A8_MTRY(dalloc(m, &m->cos_l, rope));
   W8A8_MTRY(dalloc(m, &m->sin_l, rope));
@@ -496,7 +503,7 @@ extern "C" w8a8_status w8a8_model_calibrate(w8a8_model* m, const int32_t* tokens
   W8A8_CHECK_ARG(tokens && aligned16(tokens), W8A8_ERR_INVALID_ARG, "w8a8_model_calibrate: null or unaligned tokens");
   cudaStream_t st = as_stream(stream);
   W8A8_TRY(launch_set_int(m->d_pos, 0, st));
-  return forward_core(m, tokens, B, T, nullptr, nullptr, true, st);
+  return forward_core(m, tokens, B, T, 0, nullptr, nullptr, true, st);
 }
 
 extern "C" w8a8_status w8a8_model_prepare(w8a8_model* m, float alpha, int smooth, void* stream) {
@@ -591,7 +598,7 @@ extern "C" w8a8_status w8a8_decoder_forward(w8a8_model* m, const int32_t* tokens
                  "w8a8_decoder_forward: pointers must be 16-byte aligned");
   cudaStream_t st = as_stream(stream);
   W8A8_TRY(launch_set_int(m->d_pos, start_pos, st));
-  return forward_core(m, tokens, B, T, logits, top1, false, st);
+  return forward_core(m, tokens, B, T, start_pos, logits, top1, false, st);
 }
 
 extern "C" w8a8_status w8a8_decoder_decode_step(w8a8_model* m, const int32_t* tokens, int B, int pos, float* logits,
@@ -605,7 +612,7 @@ extern "C" w8a8_status w8a8_decoder_decode_step(w8a8_model* m, const int32_t* to
   W8A8_TRY(launch_set_int(m->d_pos, pos, st));
   const int want_logits = logits != nullptr;
   if (m->trace_on) {  // traced steps run eagerly (a cached graph holds no trace copies)
-    W8A8_TRY(forward_core(m, m->d_tokens, B, 1, want_logits ? m->d_logits : nullptr, m->d_top1, false, st));
+    W8A8_TRY(forward_core(m, m->d_tokens, B, 1, pos, want_logits ? m->d_logits : nullptr, m->d_top1, false, st));
     W8A8_CUDA(cudaMemcpyAsync(top1, m->d_top1, sizeof(int32_t) * B, cudaMemcpyDeviceToDevice, st));
     if (logits)
       W8A8_CUDA(cudaMemcpyAsync(logits, m->d_logits, sizeof(float) * B * (size_t)m->cfg.vocab,
@@ -620,10 +627,10 @@ extern "C" w8a8_status w8a8_decoder_decode_step(w8a8_model* m, const int32_t* to
   if (it == m->graphs.end()) {
     // one eager step first: every lazily set kernel attribute exists before capture; it computes
     // exactly what the graph computes (same cache position, same outputs)
-    W8A8_TRY(forward_core(m, m->d_tokens, B, 1, want_logits ? m->d_logits : nullptr, m->d_top1, false, st));
+    W8A8_TRY(forward_core(m, m->d_tokens, B, 1, pos, want_logits ? m->d_logits : nullptr, m->d_top1, false, st));
     cudaGraph_t g = nullptr;
     W8A8_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    const w8a8_status s = forward_core(m, m->d_tokens, B, 1, want_logits ? m->d_logits : nullptr, m->d_top1, false, st);
+    const w8a8_status s = forward_core(m, m->d_tokens, B, 1, pos, want_logits ? m->d_logits : nullptr, m->d_top1, false, st);
     const cudaError_t e = cudaStreamEndCapture(st, &g);
     W8A8_TRY(s);
     W8A8_CUDA(e);

@@ -1,0 +1,51 @@
+"""Prefill attention on the tensor cores against the oracle decoder (two layers, one global and one with
+a window shorter than a key tile): query blocks and key tiles with ragged ends, one and two CTAs per
+query block, a second CTA without keys, and prompts fed in chunks that start at any position."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from oracle import decoder as OD
+from oracle import masks as OM
+
+pytestmark = pytest.mark.gpu
+
+L, H, F, V, WINDOW, SEQ = 2, 1152, 256, 1024, 100, 320
+
+
+@pytest.fixture(scope="module")
+def setup():
+    from paper_2608_28003_gb300 import build
+    build.build()
+    from paper_2608_28003_gb300 import binding as B
+    f32, bf, norms = synth.decoder_weights(L, H, F, V, seed=9)
+    w = {k: [t.cuda() for t in v] if isinstance(v, list) else v.cuda() for k, v in bf.items()}
+    n = {k: [torch.from_numpy(a).cuda() for a in v] if isinstance(v, list) else torch.from_numpy(v).cuda()
+         for k, v in norms.items()}
+    cfg = B.DecoderConfig(layers=L, inter=F, vocab=V, window=WINDOW, global_layers=(0,), max_batch=8, max_seq=SEQ,
+                          max_tokens=8 * SEQ)
+    ow = dict(f32)
+    ow.update(norms)
+    ocfg = OD.DecoderConfig(layers=L, inter=F, vocab=V, window=WINDOW, global_layers=(0,))
+    toks = synth.tokens(8 * 300, V, seed=4).reshape(8, 300)
+    od = OD.OracleDecoder(ocfg, ow, batch=8, max_len=SEQ)
+    ref = od.forward(toks, 0, OM.make_mask())["logits"]
+    return B.Decoder(cfg, w, n), toks, ref
+
+
+@pytest.mark.parametrize("batch,chunks", [(8, [300]),            # 96 query blocks: one CTA each
+                                          (1, [257]), (2, [128]), (1, [2]),
+                                          (2, [37, 130, 3]),     # keys of earlier calls, unaligned starts
+                                          (1, [129, 127, 44])])
+def test_chunked_prefill_matches_oracle(setup, batch, chunks):
+    dec, toks, ref = setup
+    t = torch.from_numpy(toks[:batch]).cuda()
+    pos = 0
+    for c in chunks:
+        logits, top1 = dec.forward(t[:, pos:pos + c].clone(memory_format=torch.contiguous_format), pos)
+        got = logits.view(batch, c, V).cpu().numpy().astype(np.float64)
+        want = ref[:batch, pos:pos + c]
+        rel = np.linalg.norm(got - want, axis=-1) / np.linalg.norm(want, axis=-1)
+        assert rel.max() <= 1e-2, (pos, float(rel.max()))  # the decoder's stated tolerance, all bf16
+        pos += c
