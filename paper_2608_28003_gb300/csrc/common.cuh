@@ -262,6 +262,68 @@ enum DevErr : unsigned int { DEVERR_CONSUMER_WAIT = 1u, DEVERR_PRODUCER_WAIT = 2
 constexpr size_t kErrWordOffset = 36864;
 constexpr long long kWaitBudgetCycles = 4000000000LL;  // ~2 s at 2 GHz
 
+// ------------------------------------------------------------------------ packed fp32
+// Two fp32 values in one 64-bit register: each half of a packed operation is one IEEE operation,
+// rounded to nearest even.  A packed multiply feeding a packed add is contracted into one fused
+// operation whatever the rounding modifier says, so f2_mul adds a -0 that the compiler cannot know
+// (f2_neg_zero: gridDim.z is 1 in every launch); a b + (-0) is the rounded product, signs included.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 f2_pack(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};\n" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;\n" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 f2_both(uint32_t bits) { return ((f32x2)bits << 32) | bits; }
+__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+__device__ __forceinline__ f32x2 f2_neg_zero() { return f2_both(0x7fffffffu + gridDim.z); }
+__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b, f32x2 neg_zero) { return f2_fma(a, b, neg_zero); }
+
+// ------------------------------------------------------------------------ INT8 codes
+// Codes rint(fl(x_hat r)) of two values (Eq. xint8) as an fp16 pair: the fp32 sum of the product and
+// 1.5 2^23 rounds it to the nearest integer, ties to even, and its low bits (`shifted`) are the code.
+// With r = fl(127 / max |x_hat|) a finite product rounds into [-127, 127] and needs no clamp; `bad`
+// becomes NaN when a product is NaN or infinite (NaN input, or r infinite for a row of tiny
+// values), and the caller then redoes the row by integer conversion, which maps NaN to 0 and clamps.
+constexpr uint32_t kCodeMagic = 0x4b400000u;  // 1.5 2^23
+__device__ __forceinline__ uint32_t code_pair(f32x2 xh, f32x2 r2, f32x2 nz, f32x2& bad, f32x2& shifted) {
+  const f32x2 p = f2_mul(xh, r2, nz);
+  bad = f2_fma(p, 0ull, bad);
+  shifted = f2_add(p, f2_both(kCodeMagic));
+  float a, b;
+  uint32_t h;
+  f2_unpack(f2_add(shifted, f2_both(kCodeMagic | 0x80000000u)), a, b);
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;\n" : "=r"(h) : "f"(b), "f"(a));
+  return h;
+}
+// The codes of four such pairs as bytes.
+__device__ __forceinline__ uint2 code_bytes(const f32x2 (&s)[4]) {
+  uint32_t w[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t a = __byte_perm((uint32_t)s[2 * h], (uint32_t)(s[2 * h] >> 32), 0x0040u);
+    const uint32_t b = __byte_perm((uint32_t)s[2 * h + 1], (uint32_t)(s[2 * h + 1] >> 32), 0x0040u);
+    w[h] = __byte_perm(a, b, 0x5410u);
+  }
+  return make_uint2(w[0], w[1]);
+}
+// Two integer codes as an fp16 pair.
+__device__ __forceinline__ uint32_t f16_codes(int lo, int hi) {
+  return (uint32_t)int_to_f16_bits(lo) | ((uint32_t)int_to_f16_bits(hi) << 16);
+}
+
 // --------------------------------------------------------------------- GeGLU fp32 recipe
 // gelu_tanh(g) = g / (1 + 2^w), w = -2 log2(e) * sqrt(2/pi) * (g + 0.044715 g^3), each step one
 // IEEE fp32 operation rounded to nearest-even, in the order below (no contraction into FMA).
@@ -295,34 +357,6 @@ __device__ __forceinline__ float gelu_tanh_recipe(float g) {
 }
 
 __device__ __forceinline__ float geglu_recipe(float g, float u) { return __fmul_rn(gelu_tanh_recipe(g), u); }
-
-// Two fp32 values in one 64-bit register: each half of a packed operation is one IEEE operation,
-// rounded to nearest even.  A packed multiply feeding a packed add is contracted into one fused
-// operation whatever the rounding modifier says, so f2_mul adds a -0 that the compiler cannot know
-// (f2_neg_zero: gridDim.z is 1 in every launch); a b + (-0) is the rounded product, signs included.
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 f2_pack(float lo, float hi) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};\n" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void f2_unpack(f32x2 v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;\n" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f32x2 f2_both(uint32_t bits) { return ((f32x2)bits << 32) | bits; }
-__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
-__device__ __forceinline__ f32x2 f2_neg_zero() { return f2_both(0x7fffffffu + gridDim.z); }
-__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b, f32x2 neg_zero) { return f2_fma(a, b, neg_zero); }
 
 // Whether geglu_pair takes this gate: 2^-60 <= |g| <= 2^60 or +0 (an INT32 sum of 0); NaN, infinities
 // and -0 are left to geglu_recipe.

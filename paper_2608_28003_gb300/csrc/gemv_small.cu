@@ -61,11 +61,6 @@ __device__ __forceinline__ float consumer_sum(float v, float* red, int warp, int
   return t;
 }
 
-__device__ __forceinline__ uint32_t f16x2_of(float lo, float hi) {
-  uint32_t r;
-  asm("cvt.rn.f16x2.f32 %0, %1, %2;\n" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
-}
 __device__ __forceinline__ void ldm_x2(uint32_t addr, uint32_t& r0, uint32_t& r1) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];\n" : "=r"(r0), "=r"(r1) : "r"(addr));
 }
@@ -122,6 +117,8 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
   __shared__ float s_red[CW];
   __shared__ float s_red8[MT > 4 ? MT : 1][CW];  // 8 / 16-slot K1: per-token maxima of the warps
   __shared__ float s_sx[MT];
+  __shared__ uint64_t s_xbar;  // 8 / 16 slots: the activation rows' copies
+  __shared__ uint64_t s_cbar;  // the prologue's constants
   __shared__ unsigned int s_hmax[MT];  // GeGLU epilogue: per-token max |h * 1/delta| of this CTA (float bits)
 
   const SmallPlan& p = a.p;
@@ -132,9 +129,12 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
   uint64_t* full =
       reinterpret_cast<uint64_t*>(smem_raw + (ring - raw) + (size_t)S * SB + p.xbytes + p.abytes + p.rbytes);
   uint64_t* empty = full + S;
+  const uint32_t caddr = ring + (uint32_t)(S * SB + p.xbytes + p.abytes);  // the constants' offsets start here
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row0 = blockIdx.x * R;
-  if constexpr (CW != kCW) {  // the fused residual norm runs on 8 consumer warps only (not planned)
+  // the fused residual norm runs at 1-8 token slots on 8 consumer warps (no other call is planned with it)
+  constexpr bool kRn = CW == kCW && MT <= 8 && !kFp8;
+  if constexpr (!kRn) {
     if (a.has_rn) {
       if (threadIdx.x == 0) atomicOr(a.err, DEVERR_CONSUMER_WAIT);
       return;
@@ -150,6 +150,8 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
       mbar_init(smem_u32(full + s), 1);
       mbar_init(smem_u32(empty + s), CW);
     }
+    mbar_init(smem_u32(&s_xbar), 1);
+    mbar_init(smem_u32(&s_cbar), 1);
     fence_mbar_init();
   }
   __syncthreads();
@@ -157,6 +159,18 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
   // ------------------------------------------------------------------------ producer thread
   if (warp == CW) {
     if (lane != 0) return;
+    if constexpr (MT > 1) {  // the prologue's constants, which depend on no preceding kernel
+      const float* src[3] = {a.inv_delta, a.rn.w_post, a.rn.w_next};
+      int n = 0;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) n += p.coff[i] >= 0;
+      if (n) {
+        mbar_arrive_expect_tx(smem_u32(&s_cbar), (uint32_t)(n * a.K * 4));
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+          if (p.coff[i] >= 0) bulk_g2s(caddr + (uint32_t)p.coff[i], src[i], (uint32_t)(a.K * 4), smem_u32(&s_cbar));
+      }
+    }
     bool ok = true;
     int it = 0, s = 0;
     uint32_t ph = 0;
@@ -225,7 +239,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
   // weights of the fused residual norm (constants): this thread's 8 channels
   const int nvk = a.K >> 3;
   float wp[8], wn[8];
-  if (MT == 1 && a.has_rn && tid < nvk) {
+  if (kRn && MT == 1 && a.has_rn && tid < nvk) {
     const float4* p0 = reinterpret_cast<const float4*>(a.rn.w_post + 8 * tid);
     const float4* p1 = reinterpret_cast<const float4*>(a.rn.w_next + 8 * tid);
     const float4 a0 = p0[0], a1 = p0[1], b0 = p1[0], b1 = p1[1];
@@ -234,6 +248,15 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
   }
   pdl_wait();
   uint8_t* xsp = smem_raw + (xs - raw);
+  // constant i of the prologue, from shared memory where it was copied
+  bool have_c = false;
+  auto constant = [&](int i, const float* global) -> const float* {
+    if (p.coff[i] < 0) return global;
+    if (!have_c && !mbar_wait_warp(smem_u32(&s_cbar), 0u, kWaitBudgetCycles) && lane == 0)
+      atomicOr(a.err, DEVERR_CONSUMER_WAIT);
+    have_c = true;
+    return reinterpret_cast<const float*>(smem_raw + (caddr - raw) + p.coff[i]);
+  };
   // The bf16 rows behind the activations: the caller's X, or the fused residual norm's output
   // (thread t < K / 8 owns channels 8t .. 8t+7 of every token, as in the residual-norm kernel).
   const uint16_t* xrows = a.X;
@@ -241,7 +264,32 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
   // elements between the activation rows in shared memory (bf16, or the fp16 codes of the W8A8
   // tensor-core path; INT8 codes otherwise): padded on the tensor-core paths against bank conflicts
   const int xsb = kMma ? kpad + (kQ ? 16 : 8) : kpad;
-  if (a.has_rn) {
+  // 8 / 16 slots: the rows come by bulk copies, all in flight at once, into the places the MMA reads
+  // (W8A8, FP8: the quantiser turns them into codes there).  Through registers, four loads per thread at a
+  // time, the bf16 FFN block at 8 tokens took 15.2 us, now 13.4.
+  const bool copied = kMma && !(kRn && a.has_rn);
+  if constexpr (kMma) {
+    if (copied) {
+      if (tid == 0) {
+        mbar_arrive_expect_tx(smem_u32(&s_xbar), (uint32_t)(a.M * a.K * 2));
+        for (int m = 0; m < a.M; ++m)
+          bulk_g2s(xs + (uint32_t)(m * xsb * 2), a.X + (size_t)m * a.K, (uint32_t)(a.K * 2), smem_u32(&s_xbar));
+      }
+      if constexpr (!kQ) {  // bf16: zeros past K and in slots >= M
+        const int t8 = (kpad - a.K) >> 3, v8 = kpad >> 3;
+        for (int i = tid; i < a.M * t8; i += CW * 32) {
+          const int m = i / t8, c = i - m * t8;
+          *reinterpret_cast<uint4*>(xsp + ((size_t)m * xsb + a.K + 8 * c) * 2) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        for (int i = tid; i < (MT - a.M) * v8; i += CW * 32) {
+          const int m = i / v8, c = i - m * v8;
+          *reinterpret_cast<uint4*>(xsp + ((size_t)(a.M + m) * xsb + 8 * c) * 2) = make_uint4(0u, 0u, 0u, 0u);
+        }
+      }
+      if (!mbar_wait_warp(smem_u32(&s_xbar), 0u, kWaitBudgetCycles) && lane == 0) atomicOr(a.err, DEVERR_CONSUMER_WAIT);
+    }
+  }
+  if (kRn && a.has_rn) {
     uint16_t* as = kQ ? reinterpret_cast<uint16_t*>(xsp + p.xbytes) : reinterpret_cast<uint16_t*>(xsp);
     const int astride = kQ ? kpad : xsb;  // elements between the rows in shared memory
     if constexpr (MT == 1) {
@@ -295,8 +343,8 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
       // l, l + 32, ...; the first kKeep of them stay in registers (K <= 1280: all), later ones are
       // read again for each pass.
       constexpr int kKeep = 5;
-      const float4* w_post = reinterpret_cast<const float4*>(a.rn.w_post);
-      const float4* w_next = reinterpret_cast<const float4*>(a.rn.w_next);
+      const float4* w_post = reinterpret_cast<const float4*>(constant(1, a.rn.w_post));
+      const float4* w_next = reinterpret_cast<const float4*>(constant(2, a.rn.w_next));
       for (int m = warp; m < MT; m += CW) {
         const bool live = m < a.M;
         const uint4* yr = reinterpret_cast<const uint4*>(a.rn.y + (size_t)m * a.K);
@@ -457,111 +505,114 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
           }
         }
       }
-    } else {  // eight token slots: the whole block on all tokens at once, two passes over the rows
-      // pass 1: thread t smooths vectors t, t + 256, ... of every token (eight loads in flight) and
-      // keeps each token's running max |x_hat|; one block reduction gives m_t for all tokens
-      const float4* idl = reinterpret_cast<const float4*>(a.inv_delta);
-      auto smooth8 = [&](const uint4& w, const float4& d0, const float4& d1, float (&xh)[8]) {
-        xh[0] = __fmul_rn(bf16_lo(w.x), d0.x);
-        xh[1] = __fmul_rn(bf16_hi(w.x), d0.y);
-        xh[2] = __fmul_rn(bf16_lo(w.y), d0.z);
-        xh[3] = __fmul_rn(bf16_hi(w.y), d0.w);
-        xh[4] = __fmul_rn(bf16_lo(w.z), d1.x);
-        xh[5] = __fmul_rn(bf16_hi(w.z), d1.y);
-        xh[6] = __fmul_rn(bf16_lo(w.w), d1.z);
-        xh[7] = __fmul_rn(bf16_hi(w.w), d1.w);
+    } else {
+      // 8 or 16 token slots: a warp (two of 16) per row, two short loops over its vectors, so that the
+      // rows run side by side and the code is small.  (All threads on all tokens, unrolled, was straight-line
+      // code that ran once per launch, and the warps waited for instructions: W8A8 1152 -> 6912 at 16
+      // tokens 13.8 us, now 11.1.)
+      constexpr int kRowWarps = CW >= MT ? CW / MT : 1;          // warps on one row
+      constexpr int kStep = 32 * kRowWarps;
+      const ulonglong2* idl = reinterpret_cast<const ulonglong2*>(constant(0, a.inv_delta));  // 1 / delta, two pairs each
+      const f32x2 nz = f2_neg_zero();
+      const int part = warp % kRowWarps, vi0 = lane + 32 * part;
+      auto smooth8 = [&](const uint4& w, int vi, f32x2 (&xh)[4]) {  // x_hat of vector vi, rounded products
+        const ulonglong2 d0 = idl[2 * vi], d1 = idl[2 * vi + 1];
+        xh[0] = f2_mul(f2_pack(bf16_lo(w.x), bf16_hi(w.x)), d0.x, nz);
+        xh[1] = f2_mul(f2_pack(bf16_lo(w.y), bf16_hi(w.y)), d0.y, nz);
+        xh[2] = f2_mul(f2_pack(bf16_lo(w.z), bf16_hi(w.z)), d1.x, nz);
+        xh[3] = f2_mul(f2_pack(bf16_lo(w.w), bf16_hi(w.w)), d1.y, nz);
       };
-      // tokens m0 .. m0 + 7 of vector vi (eight loads in flight; 16 slots take two groups)
-      auto load_tokens = [&](int vi, int m0, uint4 (&w)[8]) {
+      auto unpack8 = [](const f32x2 (&v)[4], float (&x)[8]) {
 #pragma unroll
-        for (int m = 0; m < 8; ++m)
-          w[m] = m0 + m < a.M ? reinterpret_cast<const uint4*>(xrows + (size_t)(m0 + m) * xstride)[vi]
-                              : make_uint4(0u, 0u, 0u, 0u);
+        for (int e = 0; e < 4; ++e) f2_unpack(v[e], x[2 * e], x[2 * e + 1]);
       };
-      float am[MT];
+#pragma unroll 1
+      for (int m = warp / kRowWarps; m < MT; m += CW / kRowWarps) {
+        const bool live = m < a.M;
+        const uint4* src = copied ? reinterpret_cast<const uint4*>(xsp + (size_t)m * xsb * 2)
+                                  : reinterpret_cast<const uint4*>(xrows + (size_t)m * xstride);
+        float mx = 0.0f;
+        if (live && a.rowmax_in) {  // the producer's partial maxima (of the same fp32 products)
+          for (int i = lane; i < a.rowmax_n; i += 32) mx = fmaxf(mx, a.rowmax_in[(size_t)i * MT + m]);
+        } else if (live) {
+#pragma unroll 4
+          for (int vi = vi0; vi < nvec; vi += kStep) {
+            f32x2 xh[4];
+            float x[8];
+            smooth8(src[vi], vi, xh);
+            unpack8(xh, x);
 #pragma unroll
-      for (int m = 0; m < MT; ++m) am[m] = 0.0f;
-      if (a.rowmax_in) {  // the producer's partial maxima stand for pass 1 (the same fp32 products)
-        for (int i = tid; i < a.rowmax_n; i += CW * 32)
-#pragma unroll
-          for (int m = 0; m < MT; ++m) am[m] = fmaxf(am[m], a.rowmax_in[(size_t)i * MT + m]);
-      }
-      for (int vi = a.rowmax_in ? nvec : tid; vi < nvec; vi += CW * 32) {
-        const float4 d0 = idl[2 * vi], d1 = idl[2 * vi + 1];
-#pragma unroll
-        for (int m0 = 0; m0 < MT; m0 += 8) {
-          uint4 w[8];
-          load_tokens(vi, m0, w);
-#pragma unroll
-          for (int m = 0; m < 8; ++m) {
-            float xh[8];
-            smooth8(w[m], d0, d1, xh);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) am[m0 + m] = fmaxf(am[m0 + m], fabsf(xh[e]));
+            for (int e = 0; e < 8; ++e) mx = fmaxf(mx, fabsf(x[e]));
           }
         }
-      }
+        mx = warp_max(mx);
+        if constexpr (kRowWarps > 1) {
+          if (lane == 0) s_red8[m][part] = mx;
+          named_bar_sync(1, CW * 32);  // every warp takes one row here: MT rows of kRowWarps warps
 #pragma unroll
-      for (int m = 0; m < MT; ++m) {
-        const float v = warp_max(am[m]);
-        if (lane == 0) s_red8[m][warp] = v;
-      }
-      named_bar_sync(1, CW * 32);
-      float rr[MT];
-#pragma unroll
-      for (int m = 0; m < MT; ++m) {
-        float mx = 0.0f;
-#pragma unroll
-        for (int i = 0; i < CW; ++i) mx = fmaxf(mx, s_red8[m][i]);
-        rr[m] = mx > 0.0f ? __fdiv_rn(kQmax, mx) : 0.0f;  // fl32(127 / m_t)
-        if (tid == m) {
+          for (int i = 0; i < kRowWarps; ++i) mx = fmaxf(mx, s_red8[m][i]);
+        }
+        const float r = mx > 0.0f ? __fdiv_rn(kQmax, mx) : 0.0f;  // fl32(127 / m_t)
+        if (lane == 0 && part == 0) {
           const float sx = __fdiv_rn(mx, kQmax);  // s_t^x = fl32(m_t / 127); 0 for slots >= M
           s_sx[m] = sx;
-          if (m < a.M && a.s_x_dbg && blockIdx.x == 0) a.s_x_dbg[m] = sx;
+          if (live && a.s_x_dbg && blockIdx.x == 0) a.s_x_dbg[m] = sx;
         }
-      }
-      // pass 2: the rows again (L1), quantised; codes of slots >= M are zeros
-      for (int vi = tid; vi < nvec; vi += CW * 32) {
-        const float4 d0 = idl[2 * vi], d1 = idl[2 * vi + 1];
-#pragma unroll
-        for (int m0 = 0; m0 < MT; m0 += 8) {
-          uint4 w8[8];
-          load_tokens(vi, m0, w8);
-#pragma unroll
-          for (int mi = 0; mi < 8; ++mi) {
-          const int m = m0 + mi;
-          float xh[8];
-          smooth8(w8[mi], d0, d1, xh);
+        uint4* dst = reinterpret_cast<uint4*>(xsp + (size_t)m * xsb * 2);
+        uint2* dbg = live && a.xq_dbg && blockIdx.x == 0 ? reinterpret_cast<uint2*>(a.xq_dbg + (size_t)m * a.K) : nullptr;
+        if (!live) {  // codes of slots >= M are zeros
+          for (int vi = vi0; vi < nvec; vi += kStep) dst[vi] = make_uint4(0u, 0u, 0u, 0u);
+          continue;
+        }
+        f32x2 bad = 0ull;  // stays 0 unless a product is NaN or infinite
+        const f32x2 r2 = f2_pack(r, r);
+#pragma unroll 4
+        for (int vi = vi0; vi < nvec; vi += kStep) {  // the row again, quantised
+          f32x2 xh[4];
+          smooth8(src[vi], vi, xh);  // copied rows: overwritten by the same lane below
           if constexpr (kFp8) {  // e4m3 codes: their fp16 values for the MMA, the bytes for debugging
             uint32_t c[4];
+            float x[8];
+            unpack8(xh, x);
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-              c[e] = e4m3x2_of(__fmul_rn(xh[2 * e], rr[m]), __fmul_rn(xh[2 * e + 1], rr[m]));
-            reinterpret_cast<uint4*>(xsp + (size_t)m * xsb * 2)[vi] =
+            for (int e = 0; e < 4; ++e) c[e] = e4m3x2_of(__fmul_rn(x[2 * e], r), __fmul_rn(x[2 * e + 1], r));
+            dst[vi] =
                 make_uint4(e4m3x2_to_f16x2(c[0]), e4m3x2_to_f16x2(c[1]), e4m3x2_to_f16x2(c[2]), e4m3x2_to_f16x2(c[3]));
-            if (a.xq_dbg && blockIdx.x == 0 && m < a.M)
-              reinterpret_cast<uint2*>(a.xq_dbg + (size_t)m * a.K)[vi] =
-                  make_uint2(c[0] | (c[1] << 16), c[2] | (c[3] << 16));
+            if (dbg) dbg[vi] = make_uint2(c[0] | (c[1] << 16), c[2] | (c[3] << 16));
           } else {
-            int q[8];
+            uint32_t c[4];
+            f32x2 sh[4];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) q[e] = max(-127, min(127, __float2int_rn(__fmul_rn(xh[e], rr[m]))));
-            if constexpr (kMma) {
-              reinterpret_cast<uint4*>(xsp + (size_t)m * xsb * 2)[vi] =
-                  make_uint4(f16x2_of((float)q[0], (float)q[1]), f16x2_of((float)q[2], (float)q[3]),
-                             f16x2_of((float)q[4], (float)q[5]), f16x2_of((float)q[6], (float)q[7]));
-            }
-            if (!kMma || (a.xq_dbg && blockIdx.x == 0 && m < a.M)) {
-              uint2 packed;
-              packed.x = (uint32_t)(q[0] & 0xff) | ((uint32_t)(q[1] & 0xff) << 8) | ((uint32_t)(q[2] & 0xff) << 16) |
-                         ((uint32_t)(q[3] & 0xff) << 24);
-              packed.y = (uint32_t)(q[4] & 0xff) | ((uint32_t)(q[5] & 0xff) << 8) | ((uint32_t)(q[6] & 0xff) << 16) |
-                         ((uint32_t)(q[7] & 0xff) << 24);
-              if (!kMma) reinterpret_cast<uint2*>(xsp + (size_t)m * kpad)[vi] = packed;
-              if (a.xq_dbg && blockIdx.x == 0 && m < a.M)
-                reinterpret_cast<uint2*>(a.xq_dbg + (size_t)m * a.K)[vi] = packed;
-            }
+            for (int e = 0; e < 4; ++e) c[e] = code_pair(xh[e], r2, nz, bad, sh[e]);
+            dst[vi] = make_uint4(c[0], c[1], c[2], c[3]);
+            if (dbg) dbg[vi] = code_bytes(sh);
           }
+        }
+        if constexpr (kInt8) {
+          float b0, b1;
+          f2_unpack(bad, b0, b1);
+          if (b0 + b1 != 0.0f) {  // NaN input, or r infinite: this lane's vectors through the integer conversion
+            const uint4* again = copied ? reinterpret_cast<const uint4*>(a.X + (size_t)m * a.K) : src;
+#pragma unroll 1
+            for (int vi = vi0; vi < nvec; vi += kStep) {
+              f32x2 xh[4];
+              float x[8];
+              int q[8];
+              smooth8(again[vi], vi, xh);
+              unpack8(xh, x);
+#pragma unroll
+              for (int e = 0; e < 8; ++e) q[e] = max(-127, min(127, __float2int_rn(__fmul_rn(x[e], r))));
+              dst[vi] = make_uint4(f16_codes(q[0], q[1]), f16_codes(q[2], q[3]), f16_codes(q[4], q[5]),
+                                   f16_codes(q[6], q[7]));
+              if (dbg) {
+                uint2 packed;
+                packed.x = (uint32_t)(q[0] & 0xff) | ((uint32_t)(q[1] & 0xff) << 8) | ((uint32_t)(q[2] & 0xff) << 16) |
+                           ((uint32_t)(q[3] & 0xff) << 24);
+                packed.y = (uint32_t)(q[4] & 0xff) | ((uint32_t)(q[5] & 0xff) << 8) | ((uint32_t)(q[6] & 0xff) << 16) |
+                           ((uint32_t)(q[7] & 0xff) << 24);
+                dbg[vi] = packed;
+              }
+            }
           }
         }
       }
@@ -579,7 +630,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
         *reinterpret_cast<uint4*>(xsp + (size_t)m * kpad + a.K + 16 * c) = make_uint4(0u, 0u, 0u, 0u);
       }
     }
-  } else if (!a.has_rn) {
+  } else if (!kMma && !a.has_rn) {
     const int vpr = kpad >> 3;  // 16-byte vectors per slot
     const int total = MT * vpr;
     for (int i0 = tid; i0 < total; i0 += 4 * CW * 32) {  // four loads in flight per thread
@@ -948,7 +999,8 @@ w8a8_status launch_t(const SmallArgs& a, cudaStream_t st) {
     W8A8_TRY(make_tmap_2d(&tw, a.W, EB, (uint64_t)a.K, (uint64_t)a.N, (uint64_t)a.K * EB, 128 / EB, 8 * RW, 128));
   else
     W8A8_TRY(make_tmap_2d(&tw, a.W, EB, (uint64_t)a.K, (uint64_t)a.N, (uint64_t)a.K * EB, 256, 8 * RW, 0));
-  W8A8_CUDA(launch_pdl(gemv_small_kernel<kW, MT, RW, CW>, dim3(a.p.P), dim3((CW + 1) * 32), (size_t)a.p.smem_bytes, st,
+  W8A8_CUDA(launch_pdl(gemv_small_kernel<kW, MT, RW, CW>, dim3(a.p.P), dim3((CW + 1) * 32),
+                       (size_t)(a.p.smem_bytes + a.p.cextra), st,
                        tw, a));
   return W8A8_OK;
 }
@@ -1048,6 +1100,22 @@ SmallPlan make_small_plan(int wkind, int M, int N, int K, int kind, int sm_count
   }
   if (p.ks == 0) return p;
   p.smem_bytes = 1024 + p.stages * p.stage_bytes + p.xbytes + p.abytes + p.rbytes + 16 * p.stages;
+  // the prologue's constants: first into the partial sums' place, then past the end as far as the SM's
+  // CTAs leave room
+  const bool want[3] = {mma && int8_weights, fused_norm && p.MT > 1, fused_norm && p.MT > 1};
+  int used = 0;
+  for (int i = 0; i < 3; ++i) {
+    p.coff[i] = -1;
+    if (!want[i]) continue;
+    const int bytes = K * 4;
+    if (used + bytes <= p.rbytes) {
+      p.coff[i] = used;
+      used += bytes;
+    } else if (cps * (p.smem_bytes + p.cextra + bytes + kStatic) <= kSmemLimit) {
+      p.coff[i] = p.rbytes + 16 * p.stages + p.cextra;
+      p.cextra += bytes;
+    }
+  }
   p.ok = 1;
   return p;
 }

@@ -28,6 +28,14 @@ struct SmallPlan {
   int rbytes;       // 5-8 tokens (tensor-core paths): the consumer warps' partial sums
   int smem_bytes;
   int cw;           // consumer warps: 8, or 16 on the tensor-core paths when the grid has one CTA per SM
+  // per-channel constants of the prologue (1 / delta; w_post and w_next of the fused residual norm), copied
+  // to shared memory before the wait for the preceding kernel (read from global memory after it, the
+  // norm weights put two more L2 latencies into q/k/v and gate/up: decode of 8 sequences 1050 us, now
+  // 939): byte offset of each behind the ring and
+  // the activations (in the partial sums' place, free until the end, or past smem_bytes), -1: read
+  // from global memory
+  int coff[3];
+  int cextra;       // dynamic shared memory past smem_bytes
 };
 
 // The decoder's residual step in front of a decode linear, fused into the GEMV's prologue:
