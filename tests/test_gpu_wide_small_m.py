@@ -1,0 +1,33 @@
+"""lm_head-sized outputs at few tokens on the tensor-core GEMM: bf16 from one token, W8A8 from 17, on both
+sides of the line and at a ragged vocabulary, logits and top-1 against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from oracle import blocks as OB
+from oracle import w8a8 as OW
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("vocab", [16400, 20000])
+@pytest.mark.parametrize("M", [1, 2, 7, 16, 17, 33, 63])
+def test_wide_output_few_tokens(M, vocab):
+    from paper_2608_28003_gb300 import build
+    build.build()
+    from paper_2608_28003_gb300 import binding as B
+    c = synth.lm_head_case(M, seed=M, hidden=1040, vocab=vocab, calib_rows=32)
+    stat = OW.act_absmax(c["calib32"])
+    w = c["w"].cuda()
+    hd = B.HeadWeights(vocab, 1040, B.prepare_weights(w, torch.from_numpy(stat).cuda(), want_f16=True), w)
+    logits, top1 = B.lm_head(hd, B.W8A8_PREC_W8A8, c["x"].cuda())
+    r = OB.lm_head_w8a8(c["x32"], OW.prepare_weights(c["w32"], stat))
+    assert np.array_equal(logits.cpu().numpy().view(np.uint32), r["logits"].view(np.uint32))
+    assert np.array_equal(top1.cpu().numpy(), r["top1"])
+    logits, top1 = B.lm_head(hd, B.W8A8_PREC_BF16, c["x"].cuda())
+    r = OB.lm_head_bf16(c["x32"], c["w32"])
+    mag = np.abs(c["x32"]).astype(np.float64) @ np.abs(c["w32"]).astype(np.float64).T
+    lg = logits.cpu().numpy()
+    assert np.all(np.abs(lg - r["logits"]) <= 1040 * 2.0 ** -24 * mag + 1e-30)  # fp32 sums, any order
+    assert np.array_equal(top1.cpu().numpy(), lg.argmax(axis=1))
