@@ -429,4 +429,16 @@ __device__ __forceinline__ uint32_t float_order_key(float v) {
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
+// The value behind a key's upper half (the inverse of float_order_key); NaN for the empty key.
+__device__ __forceinline__ float key_value(unsigned long long key) {
+  const uint32_t k = (uint32_t)(key >> 32);
+  return __uint_as_float((k & 0x80000000u) ? k ^ 0x80000000u : ~k);
+}
+// max that is NaN when an operand is
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;\n" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 }  // namespace w8a8

@@ -186,18 +186,6 @@ struct Top {
   float known;
   unsigned long long best;
 };
-// The value behind a key's upper half (the inverse of float_order_key); NaN for the empty key.
-__device__ __forceinline__ float key_value(unsigned long long key) {
-  const uint32_t k = (uint32_t)(key >> 32);
-  return __uint_as_float((k & 0x80000000u) ? k ^ 0x80000000u : ~k);
-}
-// max that is NaN when an operand is
-__device__ __forceinline__ float max_nan(float a, float b) {
-  float r;
-  asm("max.NaN.f32 %0, %1, %2;\n" : "=f"(r) : "f"(a), "f"(b));
-  return r;
-}
-
 // Chunks at .. at + n - 1 of this lane's row, kChunks 16-byte chunks wide, into the warp's block.
 template <int kChunks, int n>
 __device__ __forceinline__ void stage_row(uint32_t buf, int r, int at, const uint32_t* w) {

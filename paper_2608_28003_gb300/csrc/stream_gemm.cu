@@ -91,15 +91,26 @@ __global__ void __launch_bounds__(kThreads, Cps<NB>::value)
   constexpr int XBOX = TOK * 128;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ int s_flag;
+  __shared__ uint64_t s_xbar;  // the resident token rows
   __shared__ unsigned long long s_best[kConsumerWarps][TOK];  // top-1: per-warp best key per token slot
 
   const StreamPlan& p = a.p;
-  const int S = p.stages, SB = p.stage_bytes;
+  // The ring's slots hold one weight box (128 rows x 128 bytes) and its token boxes: half a stage of the
+  // plan, so that copies start again as soon as half a unit is consumed, and a last box wholly past K
+  // is neither copied nor multiplied (K = 1152: 9 boxes, not 5 units of 2).
+  constexpr int NBOX = KC / BOXK, BSTEPS = BOXK / 64;  // boxes per unit, 64-k steps per box
+  // With one token group the token rows stay in shared memory (p.xres bytes, loaded once: 8 tokens 73.5
+  // -> 66.7 us); otherwise they come with every box.
+  const bool xres = p.xres > 0;
+  const int S = p.slots, SB = kBox + (xres ? 0 : BSTEPS * XBOX);
   // 128-byte swizzle repeats every 1024 bytes: align the ring to 1024
   const uint32_t raw_u32 = smem_u32(smem_raw);
   const uint32_t ring = (raw_u32 + 1023u) & ~1023u;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + (ring - raw_u32) + (size_t)S * SB);
+  const uint32_t xall = ring + (uint32_t)(S * SB);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + (ring - raw_u32) + (size_t)S * SB + p.xres);
   uint64_t* empty = full + S;
+  const int kboxes = (a.K + BOXK - 1) / BOXK;  // of a row group's whole k range
+  auto boxes_of = [&](long long u) { return min(NBOX, kboxes - (int)(u % p.C) * NBOX); };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = p.G, C = p.C, Z = p.Z;
@@ -122,6 +133,7 @@ __global__ void __launch_bounds__(kThreads, Cps<NB>::value)
       mbar_init(smem_u32(full + s), 1);
       mbar_init(smem_u32(empty + s), kConsumerWarps);
     }
+    mbar_init(smem_u32(&s_xbar), 1);
     fence_mbar_init();
   }
   __syncthreads();
@@ -133,48 +145,54 @@ __global__ void __launch_bounds__(kThreads, Cps<NB>::value)
   // ------------------------------------------------------------------------ producer thread
   if (warp == kConsumerWarps) {
     if (lane != 0) return;
-    constexpr int nw = KC / BOXK, nx = KC / 64;
-    const uint32_t tx = (uint32_t)(nw * kBox + nx * XBOX);
+    const uint32_t tx = (uint32_t)SB;
     bool ok = true;
-    long long it = 0;
-    // The weights of the first stages do not depend on the preceding kernel: request them before
-    // waiting for it, then add the token rows of X to the same stages.
-    const long long npre = (long long)S < u1 - u0 ? (long long)S : u1 - u0;
-    for (; it < npre; ++it) {
-      const long long u = u0 + it;
-      const int zg = (int)(u / C), ch = (int)(u % C);
-      const int g = zg % G;
-      const uint32_t bar = smem_u32(full + (int)it);
+    long long it = 0;  // boxes issued
+    auto copy_w = [&](long long u, int h, int slot) {
+      const int zg = (int)(u / C), ch = (int)(u % C), g = zg % G;
+      const uint32_t bar = smem_u32(full + slot);
       mbar_arrive_expect_tx(bar, tx);
-      for (int b = 0; b < nw; ++b)
-        tma_load_2d(ring + (uint32_t)it * SB + b * kBox, &tmW, ch * KC + b * BOXK, g * 128, bar);
-    }
+      tma_load_2d(ring + (uint32_t)slot * SB, &tmW, ch * KC + h * BOXK, g * 128, bar);
+    };
+    auto copy_x = [&](long long u, int h, int slot) {
+      const int zg = (int)(u / C), ch = (int)(u % C), z = zg / G;
+      const uint32_t bar = smem_u32(full + slot);
+#pragma unroll
+      for (int b = 0; b < BSTEPS; ++b)
+        tma_load_2d(ring + (uint32_t)slot * SB + kBox + b * XBOX, &tmX, ch * KC + h * BOXK + b * 64, z * TOK, bar);
+    };
+    // The weights of the first slots do not depend on the preceding kernel: request them before
+    // waiting for it, then add the token rows of X to the same slots.
+    int npre = 0;
+    for (long long u = u0; u < u1 && npre < S; ++u)
+      for (int h = 0; h < boxes_of(u) && npre < S; ++h) copy_w(u, h, npre++);
     pdl_wait();
-    for (long long j = 0; j < npre; ++j) {
-      const long long u = u0 + j;
-      const int zg = (int)(u / C), ch = (int)(u % C);
-      const int z = zg / G;
-      const uint32_t bar = smem_u32(full + (int)j);
-      for (int b = 0; b < nx; ++b)
-        tma_load_2d(ring + (uint32_t)j * SB + 2 * kBox + b * XBOX, &tmX, ch * KC + b * 64, z * TOK, bar);
+    if (xres) {
+      mbar_arrive_expect_tx(smem_u32(&s_xbar), (uint32_t)p.xres);
+      for (int b = 0; b < p.xres / XBOX; ++b) tma_load_2d(xall + b * XBOX, &tmX, 64 * b, 0, smem_u32(&s_xbar));
     }
-    for (long long u = u0 + npre; u < u1; ++u, ++it) {
-      const int s = (int)(it % S);
-      const uint32_t ph = (uint32_t)((it / S) & 1);
-      if (!mbar_wait_bounded(smem_u32(empty + s), ph ^ 1u, kWaitBudgetCycles)) {
-        ok = false;
-        break;
+    int slot = 0;
+    uint32_t ph = 0;
+    for (long long u = u0; u < u1 && ok; ++u) {
+      const int nb = boxes_of(u);
+      for (int h = 0; h < nb; ++h, ++it) {
+        if (it >= npre) {
+          if (!mbar_wait_bounded(smem_u32(empty + slot), ph ^ 1u, kWaitBudgetCycles)) {
+            ok = false;
+            break;
+          }
+          copy_w(u, h, slot);
+        }
+        if (!xres) copy_x(u, h, slot);
+        if (++slot == S) {
+          slot = 0;
+          ph ^= 1u;
+        }
       }
-      const int zg = (int)(u / C), ch = (int)(u % C);
-      const int z = zg / G, g = zg % G;
-      const uint32_t bar = smem_u32(full + s);
-      const uint32_t sb = ring + (uint32_t)s * SB;
-      mbar_arrive_expect_tx(bar, tx);
-      for (int b = 0; b < nw; ++b) tma_load_2d(sb + b * kBox, &tmW, ch * KC + b * BOXK, g * 128, bar);
-      for (int b = 0; b < nx; ++b) tma_load_2d(sb + 2 * kBox + b * XBOX, &tmX, ch * KC + b * 64, z * TOK, bar);
     }
     if (!ok) atomicOr(a.err, DEVERR_PRODUCER_WAIT);
     // Let the copies of the last stages land before this CTA can exit (bounded).
+    if (xres && !mbar_wait_bounded(smem_u32(&s_xbar), 0u, kWaitBudgetCycles)) atomicOr(a.err, DEVERR_DRAIN_WAIT);
     for (long long j = it > S ? it - S : 0; j < it; ++j) {
       if (!mbar_wait_bounded(smem_u32(full + (int)(j % S)), (uint32_t)((j / S) & 1), kWaitBudgetCycles)) {
         atomicOr(a.err, DEVERR_DRAIN_WAIT);
@@ -223,74 +241,99 @@ __global__ void __launch_bounds__(kThreads, Cps<NB>::value)
     best_z = -1;
   };
 
-  // dequantised (or bf16-path) fp32 value of an accumulator, before the bias
-  auto value_f32 = [&](uint32_t v, int i, int tk) -> float {
+  const bool want_top = a.kind == EPI_F32 && a.top1 != nullptr;
+  // Largest logit seen for this lane's tokens (those of lane t = lane & 3): only a row block that
+  // reaches it goes through the 64-bit keys.
+  float known[NB][2];
+#pragma unroll
+  for (int nb = 0; nb < NB; ++nb) known[nb][0] = known[nb][1] = -INFINITY;
+  // Scales and biases of the lane's two rows: read when the row group begins, so that their latency (a
+  // scale vector of lm_head size comes from HBM) passes under its products (read in the epilogue: W8A8 lm_head at 16 tokens 80.6 us, now
+  // 74.0; at 8 tokens 66.7, now 62.4).
+  float swa = 0.0f, swb = 0.0f, ba = 0.0f, bb = 0.0f;
+  auto load_rows = [&](int g) {
+    const int ra = g * 128 + 16 * w + pr, rb = ra + 8;
     if constexpr (kInt8) {
-      const float sc = __fmul_rn(a.s_x[tk], a.s_w[i]);  // s_t^x * s_i^W
-      return __fmul_rn(sc, __int2float_rn((int)v));
-    } else {
-      return __uint_as_float(v);
+      swa = ra < a.N ? a.s_w[ra] : 0.0f;
+      swb = rb < a.N ? a.s_w[rb] : 0.0f;
+    }
+    if (a.bias) {
+      ba = ra < a.N ? a.bias[ra] : 0.0f;
+      bb = rb < a.N ? a.bias[rb] : 0.0f;
     }
   };
-
-  const bool want_top = a.kind == EPI_F32 && a.top1 != nullptr;
   auto epilogue = [&](int z, int g, uint32_t (&v)[NB][4]) {
     const int ra = g * 128 + 16 * w + pr, rb = ra + 8;
+    const bool ina = ra < a.N, inb = rb < a.N;
+    float sx[NB][2];  // the scales of the lane's tokens, read before any store
+#pragma unroll
+    for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int tk = z * TOK + nb * 8 + 2 * t + h;
+        sx[nb][h] = kInt8 && tk < a.M ? a.s_x[tk] : 0.0f;
+      }
+    // dequantised (or bf16-path) fp32 value of an accumulator (+ bias): fl(fl(s_t^x s_i^W) acc)
+    auto value = [&](uint32_t acc, float sxv, float sw, float b) -> float {
+      float y;
+      if constexpr (kInt8)
+        y = __fmul_rn(__fmul_rn(sxv, sw), __int2float_rn((int)acc));
+      else
+        y = __uint_as_float(acc);
+      return a.bias ? __fadd_rn(y, b) : y;
+    };
     if (want_top && z != best_z) {
       publish_top();
       best_z = z;
       for (int i = lane; i < TOK; i += 32) s_best[w][i] = 0ull;
+#pragma unroll
+      for (int nb = 0; nb < NB; ++nb) known[nb][0] = known[nb][1] = -INFINITY;
       __syncwarp();
     }
 #pragma unroll
     for (int nb = 0; nb < NB; ++nb) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        unsigned long long best = 0ull;
         const int tk = z * TOK + nb * 8 + 2 * t + h;
-        if (tk >= a.M) {
-        } else if (a.kind == EPI_GEGLU) {
-          if (rb >= a.N) continue;
-          float gv = value_f32(v[nb][h], ra, tk), uv = value_f32(v[nb][2 + h], rb, tk);
-          if (a.bias) {
-            gv = __fadd_rn(gv, a.bias[ra]);
-            uv = __fadd_rn(uv, a.bias[rb]);
-          }
+        const bool live = tk < a.M;
+        const float ya = value(v[nb][h], sx[nb][h], swa, ba), yb = value(v[nb][2 + h], sx[nb][h], swb, bb);
+        if (live) {
           if constexpr (kInt8) {
-            if (a.acc_dbg) {
-              a.acc_dbg[(size_t)tk * a.N + ra] = (int)v[nb][h];
-              a.acc_dbg[(size_t)tk * a.N + rb] = (int)v[nb][2 + h];
-            }
+            if (a.acc_dbg && ina) a.acc_dbg[(size_t)tk * a.N + ra] = (int)v[nb][h];
+            if (a.acc_dbg && inb) a.acc_dbg[(size_t)tk * a.N + rb] = (int)v[nb][2 + h];
           }
-          a.y[(size_t)tk * (a.N >> 1) + ((g * 128 + 16 * w) >> 1) + pr] = f32_to_bf16_bits(geglu_recipe(gv, uv));
-        } else {
+          if (a.kind == EPI_GEGLU) {
+            if (inb) a.y[(size_t)tk * (a.N >> 1) + ((g * 128 + 16 * w) >> 1) + pr] = f32_to_bf16_bits(geglu_recipe(ya, yb));
+          } else if (a.kind == EPI_BF16) {
+            if (ina) a.y[(size_t)tk * a.N + ra] = f32_to_bf16_bits(ya);
+            if (inb) a.y[(size_t)tk * a.N + rb] = f32_to_bf16_bits(yb);
+          } else if (a.logits) {
+            if (ina) a.logits[(size_t)tk * a.N + ra] = ya;
+            if (inb) a.logits[(size_t)tk * a.N + rb] = yb;
+          }
+        }
+        if (want_top) {  // over the block's 16 rows: the 8 lanes with equal t
+          float m = max_nan(live && ina ? ya : -INFINITY, live && inb ? yb : -INFINITY);
 #pragma unroll
-          for (int side = 0; side < 2; ++side) {
-            const int i = side ? rb : ra;
-            if (i >= a.N) continue;
-            const uint32_t raw = v[nb][2 * side + h];
-            float y = value_f32(raw, i, tk);
-            if (a.bias) y = __fadd_rn(y, a.bias[i]);
-            if constexpr (kInt8) {
-              if (a.acc_dbg) a.acc_dbg[(size_t)tk * a.N + i] = (int)raw;
-            }
-            if (a.kind == EPI_BF16) {
-              a.y[(size_t)tk * a.N + i] = f32_to_bf16_bits(y);
-            } else {
-              if (a.logits) a.logits[(size_t)tk * a.N + i] = y;
+          for (int o = 4; o < 32; o <<= 1) m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, o));
+          if (__any_sync(0xffffffffu, !(m < known[nb][h]))) {
+            unsigned long long best = 0ull;
+            auto offer = [&](float y, int i) {
               const unsigned long long key =
                   ((unsigned long long)float_order_key(y) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)i);
               best = key > best ? key : best;
-            }
-          }
-        }
-        if (want_top) {  // max over the 8 row pairs (lanes with equal t)
+            };
+            if (live && ina) offer(ya, ra);
+            if (live && inb) offer(yb, rb);
 #pragma unroll
-          for (int o = 4; o < 32; o <<= 1) {
-            const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
-            best = other > best ? other : best;
+            for (int o = 4; o < 32; o <<= 1) {
+              const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
+              best = other > best ? other : best;
+            }
+            const int i = nb * 8 + 2 * t + h;
+            if (gl == 0 && best > s_best[w][i]) s_best[w][i] = best;
+            if (!(m < known[nb][h])) known[nb][h] = m;
           }
-          if (gl == 0 && best > s_best[w][nb * 8 + 2 * t + h]) s_best[w][nb * 8 + 2 * t + h] = best;
         }
       }
     }
@@ -386,99 +429,103 @@ __global__ void __launch_bounds__(kThreads, Cps<NB>::value)
 
   zero_acc();
   int cur = -1, chf = 0, chl = 0;
-  long long it = 0;
   const uint32_t rowA = (uint32_t)(16 * w + pr) * 128u, rowB = rowA + 8u * 128u;
-  for (long long u = u0; u < u1; ++u, ++it) {
+  if (xres && !mbar_wait_warp(smem_u32(&s_xbar), 0u, kWaitBudgetCycles)) {
+    ok = false;
+    if (lane == 0) atomicOr(a.err, DEVERR_CONSUMER_WAIT);
+  }
+  int slot = 0;
+  uint32_t ph = 0;
+  for (long long u = u0; u < u1; ++u) {
     const int zg = (int)(u / C), ch = (int)(u % C);
     if (zg != cur) {
       if (cur >= 0) flush(cur, chf, chl);
       cur = zg;
       chf = ch;
       zero_acc();
+      load_rows(zg % G);
     }
     chl = ch;
-    const int s = (int)(it % S);
-    const uint32_t ph = (uint32_t)((it / S) & 1);
-    if (ok) {
-      bool got = true;
-      if (lane == 0) got = mbar_wait_bounded(smem_u32(full + s), ph, kWaitBudgetCycles);
-      got = __shfl_sync(0xffffffffu, got, 0);
-      if (!got) {
+    const int nbx = boxes_of(u);
+#pragma unroll 1
+    for (int h = 0; h < nbx; ++h) {
+      if (ok && !mbar_wait_warp(smem_u32(full + slot), ph, kWaitBudgetCycles)) {
         ok = false;
         if (lane == 0) atomicOr(a.err, DEVERR_CONSUMER_WAIT);
       }
-    }
-    if (!ok) continue;  // no data: skip the math and do not release the stage
-
-    const uint32_t sb = ring + (uint32_t)s * SB;
+      if (!ok) break;  // no data: skip the math and do not release the slot
+      const uint32_t sb = ring + (uint32_t)slot * SB;
 #pragma unroll
-    for (int st = 0; st < STEPS; ++st) {
-      uint4 wa[2], wb[2];
-      if constexpr (kInt8) {
-        // weight box st/2, logical 16-byte chunk 4(st%2) + t of rows pr and pr+8 (row & 7 == pr)
-        const uint32_t wbox = sb + (uint32_t)(st >> 1) * kBox;
-        const uint32_t off = (uint32_t)(((4 * (st & 1) + t) ^ pr) << 4);
-        wa[0] = lds128(wbox + rowA + off);
-        wb[0] = lds128(wbox + rowB + off);
-      } else {
-        // weight box st, logical chunks 2t and 2t+1 of rows gl and gl+8
-        const uint32_t wbox = sb + (uint32_t)st * kBox;
-        const uint32_t o0 = (uint32_t)(((2 * t) ^ pr) << 4), o1 = (uint32_t)(((2 * t + 1) ^ pr) << 4);
-        wa[0] = lds128(wbox + rowA + o0);
-        wa[1] = lds128(wbox + rowA + o1);
-        wb[0] = lds128(wbox + rowB + o0);
-        wb[1] = lds128(wbox + rowB + o1);
-      }
-      // A fragments of the four MMAs of this step (INT8 codes widened to fp16 in registers)
-      uint32_t af[4][4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
+      for (int st = 0; st < BSTEPS; ++st) {
+        uint4 wa[2], wb[2];
         if constexpr (kInt8) {
-          i8x4_to_f16x2x2(u4c(wa[0], j), af[j][0], af[j][2]);
-          i8x4_to_f16x2x2(u4c(wb[0], j), af[j][1], af[j][3]);
+          // logical 16-byte chunk 4 st + t of the weight box, rows pr and pr+8 (row & 7 == pr)
+          const uint32_t off = (uint32_t)(((4 * st + t) ^ pr) << 4);
+          wa[0] = lds128(sb + rowA + off);
+          wb[0] = lds128(sb + rowB + off);
         } else {
-          af[j][0] = u4c(wa[j >> 1], (2 * j) & 3);
-          af[j][2] = u4c(wa[j >> 1], (2 * j + 1) & 3);
-          af[j][1] = u4c(wb[j >> 1], (2 * j) & 3);
-          af[j][3] = u4c(wb[j >> 1], (2 * j + 1) & 3);
+          // logical chunks 2t and 2t+1 of rows gl and gl+8
+          const uint32_t o0 = (uint32_t)(((2 * t) ^ pr) << 4), o1 = (uint32_t)(((2 * t + 1) ^ pr) << 4);
+          wa[0] = lds128(sb + rowA + o0);
+          wa[1] = lds128(sb + rowA + o1);
+          wb[0] = lds128(sb + rowB + o0);
+          wb[1] = lds128(sb + rowB + o1);
         }
-      }
-      const uint32_t xbox = sb + 2 * kBox + (uint32_t)st * XBOX;
-#pragma unroll
-      for (int nb = 0; nb < NB; ++nb) {
-        const uint32_t xr = xbox + (uint32_t)(nb * 8 + gl) * 128u;  // token row & 7 == gl
-        const uint4 x0 = lds128(xr + (uint32_t)(((2 * t) ^ gl) << 4));
-        const uint4 x1 = lds128(xr + (uint32_t)(((2 * t + 1) ^ gl) << 4));
-#pragma unroll
+        // A fragments of the four MMAs of this step (INT8 codes widened to fp16 in registers)
+        uint32_t af[4][4];
+  #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const uint4& xv = (j >> 1) ? x1 : x0;
-          const uint32_t b0 = u4c(xv, (2 * j) & 3);
-          const uint32_t b1 = u4c(xv, (2 * j + 1) & 3);
-          if constexpr (kInt8)
-            mma_f16_16816(acc[j % CH][nb], af[j][0], af[j][1], af[j][2], af[j][3], b0, b1);
-          else
-            mma_bf16_16816(acc[j % CH][nb], af[j][0], af[j][1], af[j][2], af[j][3], b0, b1);
+          if constexpr (kInt8) {
+            i8x4_to_f16x2x2(u4c(wa[0], j), af[j][0], af[j][2]);
+            i8x4_to_f16x2x2(u4c(wb[0], j), af[j][1], af[j][3]);
+          } else {
+            af[j][0] = u4c(wa[j >> 1], (2 * j) & 3);
+            af[j][2] = u4c(wa[j >> 1], (2 * j + 1) & 3);
+            af[j][1] = u4c(wb[j >> 1], (2 * j) & 3);
+            af[j][3] = u4c(wb[j >> 1], (2 * j + 1) & 3);
+          }
+        }
+        const uint32_t xbox = (xres ? xall + (uint32_t)((ch * NBOX + h) * BSTEPS) * XBOX : sb + kBox) + (uint32_t)st * XBOX;
+  #pragma unroll
+        for (int nb = 0; nb < NB; ++nb) {
+          const uint32_t xr = xbox + (uint32_t)(nb * 8 + gl) * 128u;  // token row & 7 == gl
+          const uint4 x0 = lds128(xr + (uint32_t)(((2 * t) ^ gl) << 4));
+          const uint4 x1 = lds128(xr + (uint32_t)(((2 * t + 1) ^ gl) << 4));
+  #pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint4& xv = (j >> 1) ? x1 : x0;
+            const uint32_t b0 = u4c(xv, (2 * j) & 3);
+            const uint32_t b1 = u4c(xv, (2 * j + 1) & 3);
+            if constexpr (kInt8)
+              mma_f16_16816(acc[j % CH][nb], af[j][0], af[j][1], af[j][2], af[j][3], b0, b1);
+            else
+              mma_bf16_16816(acc[j % CH][nb], af[j][0], af[j][1], af[j][2], af[j][3], b0, b1);
+          }
         }
       }
-    }
-    if constexpr (kInt8) {
-      since += STEPS;
-      if (since >= 16) {  // 16 steps = 1024 k: every partial sum so far is below 2^24
-#pragma unroll
-        for (int nb = 0; nb < NB; ++nb)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-#pragma unroll
-            for (int c = 0; c < CH; ++c) {
-              iacc[nb][e] += __float2int_rn(acc[c][nb][e]);
-              acc[c][nb][e] = 0.0f;
+      if constexpr (kInt8) {
+        since += BSTEPS;
+        if (since >= 16) {  // 16 steps = 1024 k: every partial sum so far is below 2^24
+  #pragma unroll
+          for (int nb = 0; nb < NB; ++nb)
+  #pragma unroll
+            for (int e = 0; e < 4; ++e) {
+  #pragma unroll
+              for (int c = 0; c < CH; ++c) {
+                iacc[nb][e] += __float2int_rn(acc[c][nb][e]);
+                acc[c][nb][e] = 0.0f;
+              }
             }
-          }
-        since = 0;
+          since = 0;
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(empty + slot));
+      if (++slot == S) {
+        slot = 0;
+        ph ^= 1u;
       }
     }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(smem_u32(empty + s));
   }
   if (cur >= 0) flush(cur, chf, chl);
   if (!want_top) return;
@@ -898,7 +945,16 @@ StreamPlan make_stream_plan(bool int8_weights, int M, int N, int K, int sm_count
   }
   p.stage_bytes = stage_bytes_for(int8_weights, p.TOK);
   p.stages = std::max(2, std::min(8, (kSmemLimit / cps - kStaticReserve - 2048) / p.stage_bytes));
-  p.smem_bytes = p.stages * p.stage_bytes + 16 * p.stages + 1024;  // + alignment slack for the ring
+  // the ring: as many half stages as fit
+  const int room = kSmemLimit / cps - kStaticReserve - 2048, boxk = int8_weights ? 128 : 64;
+  int half = p.stage_bytes / 2;
+  const int xall = (K + boxk - 1) / boxk * (boxk / 64) * p.TOK * 128;  // the token rows, in whole boxes
+  if (p.Z == 1 && room - xall >= 3 * kBox) {
+    p.xres = xall;
+    half = kBox;
+  }
+  p.slots = std::min(16, (room - p.xres) / half);
+  p.smem_bytes = p.slots * half + p.xres + 16 * p.slots + 1024;  // + alignment slack for the ring
   p.partial_bytes = (size_t)p.P * 2 * 128 * p.TOK * 4;
   return p;
 }

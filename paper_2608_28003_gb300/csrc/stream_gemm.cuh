@@ -21,6 +21,8 @@ struct StreamPlan {
   int P;        // CTAs (persistent, one per SM)
   int stages;   // pipeline depth
   int stage_bytes;
+  int slots;    // ring slots of the streaming kernel: one weight box each, with its token boxes unless resident
+  int xres;     // bytes of the token rows when they stay in shared memory (one token group), else 0
   int smem_bytes;
   size_t partial_bytes;  // [P][2][128][TOK] int32/fp32
 };
