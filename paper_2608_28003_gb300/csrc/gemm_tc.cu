@@ -1197,17 +1197,20 @@ constexpr int kMinKbPerPart = 2;
 
 // The parts are also capped at K / (4 R), so that the partials a tile's last unit reads back (KS R
 // BN fp32) stay below half of the tile's weight bytes (BN K bf16), and fewer than kMinParts parts
-// are not worth the arrival protocol.  Measured: 6-8 parts on q/k/v and o at 32 tokens save 1.5 us
-// of 10-11, the down projection drops from 34 to 12-16 us, and q/k/v and o at 128 tokens (2 parts
-// under the cap) would lose.
-constexpr int kMinParts = 4;
+// are not worth the arrival protocol: the down projection (108 stages) at 64 tokens takes 10.3 us in 8
+// parts and 23.9 whole.  A short k range is over before the partials have made their round trip, which
+// grows with the rows: from 33 tokens, ranges of up to kShortStages stages stay whole (1152 -> 1536 bf16
+// at 37 tokens 9.1 us in 6 parts, 6.4 whole, at 64 tokens 8.2 / 6.4; 1024 -> 1152 at 37 tokens 8.7 / 6.1;
+// a whole range costs 0.19 us a stage, so the lines cross near 28 stages).  Up to 32 tokens the two
+// are within 0.7 us of each other (1024 -> 1152 at 17 tokens 5.8 / 6.1) and the split stays.
+constexpr int kMinParts = 4, kShortStages = 28, kSplitAnyRows = 32;
 
 // k parts of a single-CTA call on BN-column tiles (1: no split); split_ok: the caller gave the
 // partials and tile counters the split needs
 int split_parts(int mode, int M, int N, int K, int kind, bool split_ok, int bn, int sms) {
   const int nkb = (K + bk_elems(mode) - 1) / bk_elems(mode);
   const long long tiles = (long long)((N + bn - 1) / bn) * ((M + kBM - 1) / kBM);
-  if (kind == EPI_BF16 && split_ok && 2 * tiles <= sms) {
+  if (kind == EPI_BF16 && split_ok && 2 * tiles <= sms && (nkb > kShortStages || a_box_rows(M) <= kSplitAnyRows)) {
     const int ks = std::min({(int)(sms / tiles), nkb / kMinKbPerPart, K / (4 * a_box_rows(M))});
     if (ks >= kMinParts) return ks;
   }
