@@ -1,5 +1,6 @@
 // C-ABI entry points of libw8a8: argument checks, workspace carve-up and kernel dispatch for the
 // W8A8 linear, the bf16 pass-through linear, the FFN block and lm_head.
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <mutex>
@@ -163,6 +164,12 @@ bool decode_gemv_takes(bool int8, int M, int N, int K, bool geglu, int sms) {
 // 63 104 / 277; W8A8 at 17 tokens 104 / 117, at 33 107 / 276.  W8A8 at up to 16 tokens stays with the
 // streaming kernel, which reads the INT8 codes, half the bytes of their fp16 copy (16 tokens 81 / 103).
 constexpr int kTcMinTokensWideInt8 = 17, kTcMinTokensWideBf16 = 1, kTcMinTokensNarrow = 9, kTcNarrowMaxN = 16384;
+
+// Whether a bf16 lm_head call runs the tensor-core GEMM (tc_path's rule for logits).
+static bool head_bf16_on_tc(int M, int N, int K) {
+  return M >= (N <= kTcNarrowMaxN ? kTcMinTokensNarrow : kTcMinTokensWideBf16) &&
+         tc_gemm_supported(M, N, K, EPI_F32, true, max_top_keys());
+}
 
 static bool tc_path(bool int8, const void* W16, const uint16_t* X, int M, int N, int K, const float* bias, int kind,
                     const float* inv_delta, const float* s_w, uint16_t* Y, float* logits, int32_t* top1,
@@ -616,6 +623,8 @@ extern "C" w8a8_status w8a8_ffn_block(const w8a8_ffn_weights* f, int precision, 
 extern "C" w8a8_status w8a8_lm_head_workspace_size(int M, int vocab, int hidden, size_t* bytes) {
   W8A8_CHECK_ARG(bytes && M >= 0 && vocab >= 0 && hidden >= 0, W8A8_ERR_INVALID_ARG, "w8a8_lm_head_workspace_size: bad argument");
   *bytes = linear_ws(M, vocab, hidden, true, device_sms()).total;
+  // a bf16 call that the streaming kernel takes may need more for its partial sums
+  if (!head_bf16_on_tc(M, vocab, hidden)) *bytes = std::max(*bytes, linear_ws(M, vocab, hidden, false, device_sms()).total);
   return W8A8_OK;
 }
 
@@ -642,6 +651,8 @@ extern "C" w8a8_status w8a8_lm_head(const w8a8_head_weights* hd, int precision, 
     return run_w8a8_linear(&hd->q, X, M, nullptr, EPI_F32, nullptr, logits, top1, nullptr, workspace, d.sms, st);
   }
   W8A8_CHECK_ARG(hd->bf16 && aligned16(hd->bf16), W8A8_ERR_INVALID_ARG, "w8a8_lm_head: null or unaligned bf16 table");
-  W8A8_TRY(check_ws("w8a8_lm_head", workspace, ws_bytes, linear_ws(M, V, D, false, d.sms).total));
+  // the tensor-core GEMM's logits need no partial sums
+  W8A8_TRY(check_ws("w8a8_lm_head", workspace, ws_bytes,
+                    head_bf16_on_tc(M, V, D) ? (size_t)W8A8_WS_RESERVED : linear_ws(M, V, D, false, d.sms).total));
   return run_bf16_linear(hd->bf16, V, D, X, M, nullptr, EPI_F32, nullptr, logits, top1, workspace, d.sms, st);
 }
