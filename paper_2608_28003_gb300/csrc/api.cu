@@ -116,13 +116,39 @@ struct RowMax {
   int n;                        // down: gate/up's CTA count
 };
 
+constexpr int kSeparateK1MinK = 4096;  // at 5-8 tokens; between the two measured lengths 1152 and 6912
+
 static bool small_gemv(bool int8, const void* W, const float* inv_delta, const float* s_w, const uint16_t* X, int M,
                        int N, int K, const float* bias, int kind, uint16_t* Y, const w8a8_debug* dbg, void* ws,
-                       const ResNorm* rn, int sms, cudaStream_t st, w8a8_status* status, const RowMax* rm = nullptr) {
+                       const ResNorm* rn, int sms, cudaStream_t st, w8a8_status* status, const RowMax* rm = nullptr,
+                       const PreCodes* pre = nullptr, uint16_t* codes = nullptr, float* s_x = nullptr) {
   if (kind != EPI_BF16 && kind != EPI_GEGLU) return false;
   SmallArgs a{};
   a.p = make_small_plan(int8, M, N, K, kind, sms, rn != nullptr);
   if (!a.p.ok) return false;
+  // Every CTA of this kernel needs all the codes.  Where its own pass over the rows takes longer than a
+  // launch of the quantiser (one block per row, or several where the row maxima are known), that launch
+  // writes them to `codes` and `s_x`, unless the producer of X has already: W8A8 1152 -> 6912 at 16 tokens
+  // 11.0 -> 9.5 us, 6912 -> 1152 at 8 tokens 11.4 -> 9.0, the FFN block at 8 tokens 20.2 -> 18.9.  At 5-8
+  // tokens and K = 1152 the pass takes under 2 us, less than a launch (1152 -> 6912: 7.6 us with it).
+  const bool known = rm && rm->in, long_k = K >= kSeparateK1MinK;
+  if (int8 && a.p.MT >= 8 && codes && !rn && (a.p.MT == 16 || long_k)) {
+    if (pre && pre->codes16 && !dbg) {
+      a.codes = pre->codes16;
+      a.s_x = pre->s_x;
+    } else {
+      if (known)
+        *status = launch_quantize_known_rows(X, M, K, inv_delta, rm->in, rm->n, a.p.MT, codes, s_x, st);
+      else
+        *status = launch_quantize_rows(X, M, K, inv_delta, dbg ? dbg->xq : nullptr, codes, s_x, st);
+      if (*status == W8A8_OK && dbg && dbg->s_x &&
+          cudaMemcpyAsync(dbg->s_x, s_x, sizeof(float) * M, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+        *status = W8A8_ERR_CUDA;
+      if (*status != W8A8_OK) return true;
+      a.codes = codes;
+      a.s_x = s_x;
+    }
+  }
   if (rm) {
     a.rowmax_out = rm->out;
     a.next_inv_delta = rm->next_inv_delta;
@@ -230,14 +256,15 @@ w8a8_status run_w8a8_linear(const w8a8_qweight* w, const uint16_t* X, int M, con
                                    int sms, cudaStream_t st, const ResNorm* rn, const PreCodes* pre) {
   const int N = w->n, K = w->k;
   w8a8_status small_status = W8A8_OK;
-  if (!logits && !top1 &&
-      small_gemv(true, w->wq, w->inv_delta, w->s_w, X, M, N, K, bias, kind, Y, dbg, ws, rn, sms, st, &small_status))
-    return small_status;
-  W8A8_CHECK_ARG(!rn, W8A8_ERR_SHAPE, "fused residual norm: the decode GEMV does not take M=%d N=%d K=%d", M, N, K);
   LinearWs L = linear_ws(M, N, K, true, sms);
   char* base = reinterpret_cast<char*>(ws);
   void* codes = base + L.xf16;
   float* s_x = reinterpret_cast<float*>(base + L.sx);
+  if (!logits && !top1 &&
+      small_gemv(true, w->wq, w->inv_delta, w->s_w, X, M, N, K, bias, kind, Y, dbg, ws, rn, sms, st, &small_status, nullptr,
+                 pre, reinterpret_cast<uint16_t*>(codes), s_x))
+    return small_status;
+  W8A8_CHECK_ARG(!rn, W8A8_ERR_SHAPE, "fused residual norm: the decode GEMV does not take M=%d N=%d K=%d", M, N, K);
   if (tc_path(true, w->wq_f16, X, M, N, K, bias, kind, w->inv_delta, w->s_w, Y, logits, top1, dbg, ws, codes, s_x,
               base + L.part, st, &small_status, pre))
     return small_status;
@@ -469,16 +496,19 @@ w8a8_status run_ffn(const w8a8_ffn_weights* f, int precision, const uint16_t* X,
     const bool handoff = pg.ok && pd.ok && pg.MT >= 8 && pd.MT == pg.MT;
     float* rowmax = reinterpret_cast<float*>(base + L.rowmax);
     const RowMax rm_gu{rowmax, f->down.inv_delta, nullptr, 0}, rm_dn{nullptr, nullptr, rowmax, pg.P};
+    const LinearWs lg = linear_ws(M, 2 * F, H, true, sms), ld = linear_ws(M, H, F, true, sms);
+    char *gu = base + L.gu - W8A8_WS_RESERVED, *dn = base + L.dn - W8A8_WS_RESERVED;  // + a LinearWs offset
     if (small_gemv(true, f->gate_up.wq, f->gate_up.inv_delta, f->gate_up.s_w, X, M, 2 * F, H, nullptr, EPI_GEGLU, h,
-                   nullptr, workspace, rn_gate_up, sms, st, &ss, handoff ? &rm_gu : nullptr)) {
+                   nullptr, workspace, rn_gate_up, sms, st, &ss, handoff ? &rm_gu : nullptr, pre_gate_up,
+                   reinterpret_cast<uint16_t*>(gu + lg.xf16), reinterpret_cast<float*>(gu + lg.sx))) {
       W8A8_TRY(ss);
     } else if (rn_gate_up) {
       W8A8_CHECK_ARG(false, W8A8_ERR_SHAPE, "fused residual norm: the decode GEMV does not take gate/up at M=%d", M);
     } else if (tc_path(true, f->gate_up.wq_f16, X, M, 2 * F, H, nullptr, EPI_GEGLU, f->gate_up.inv_delta,
                        f->gate_up.s_w, h, nullptr, nullptr, nullptr, workspace,
-                       base + L.gu + (linear_ws(M, 2 * F, H, true, sms).xf16 - W8A8_WS_RESERVED),
-                       reinterpret_cast<float*>(base + L.gu + (linear_ws(M, 2 * F, H, true, sms).sx - W8A8_WS_RESERVED)),
-                       base + L.gu + (linear_ws(M, 2 * F, H, true, sms).part - W8A8_WS_RESERVED), st, &ss,
+                       base + L.gu + (lg.xf16 - W8A8_WS_RESERVED),
+                       reinterpret_cast<float*>(base + L.gu + (lg.sx - W8A8_WS_RESERVED)),
+                       base + L.gu + (lg.part - W8A8_WS_RESERVED), st, &ss,
                        pre_gate_up)) {
       W8A8_TRY(ss);
     } else {
@@ -502,13 +532,14 @@ w8a8_status run_ffn(const w8a8_ffn_weights* f, int precision, const uint16_t* X,
       W8A8_TRY(launch_stream_gemm(true, a, st));
     }
     if (small_gemv(true, f->down.wq, f->down.inv_delta, f->down.s_w, h, M, H, F, nullptr, EPI_BF16, Y, nullptr,
-                   workspace, nullptr, sms, st, &ss, handoff ? &rm_dn : nullptr)) {
+                   workspace, nullptr, sms, st, &ss, handoff ? &rm_dn : nullptr, nullptr,
+                   reinterpret_cast<uint16_t*>(dn + ld.xf16), reinterpret_cast<float*>(dn + ld.sx))) {
       W8A8_TRY(ss);
     } else if (tc_path(true, f->down.wq_f16, h, M, H, F, nullptr, EPI_BF16, f->down.inv_delta, f->down.s_w, Y,
                        nullptr, nullptr, nullptr, workspace,
-                       base + L.dn + (linear_ws(M, H, F, true, sms).xf16 - W8A8_WS_RESERVED),
-                       reinterpret_cast<float*>(base + L.dn + (linear_ws(M, H, F, true, sms).sx - W8A8_WS_RESERVED)),
-                       base + L.dn + (linear_ws(M, H, F, true, sms).part - W8A8_WS_RESERVED), st, &ss)) {
+                       base + L.dn + (ld.xf16 - W8A8_WS_RESERVED),
+                       reinterpret_cast<float*>(base + L.dn + (ld.sx - W8A8_WS_RESERVED)),
+                       base + L.dn + (ld.part - W8A8_WS_RESERVED), st, &ss)) {
       W8A8_TRY(ss);
     } else {
       const LinearWs B = linear_ws(M, H, F, true, sms);

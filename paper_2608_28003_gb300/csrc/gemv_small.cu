@@ -15,7 +15,8 @@
 //    memory, optionally computing them first from the decoder's residual step (residual add and
 //    the two RMSNorms, fused here instead of a separate launch).  The W8A8 path quantises them
 //    there, with the arithmetic of the stand-alone per-token quantiser (Eq. stx / xint8,
-//    smoothing of Eq. xhat-lmhead), so one launch does K1 and K3;
+//    smoothing of Eq. xhat-lmhead), so one launch does K1 and K3; at 9-16 tokens, and at 5-8 with a
+//    long K, the codes come from a launch of their own, since every CTA would repeat all that work;
 //  * warp w takes rows w, w + 8, ...; in every sub-slice lane l reads bytes 16 l .. 16 l + 15 of
 //    a row's 512 bytes (consecutive lanes read consecutive bytes: no bank conflicts);
 //  * INT8: four dp4a per 16 bytes and token, exact INT32 sums (Eq. gemm-final); bf16: fp32 FMAs,
@@ -129,6 +130,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
   uint64_t* full =
       reinterpret_cast<uint64_t*>(smem_raw + (ring - raw) + (size_t)S * SB + p.xbytes + p.abytes + p.rbytes);
   uint64_t* empty = full + S;
+  const bool pre = kInt8 && (MT == 16 || (kMma && a.codes));  // the activations come as codes: no quantiser here
   const uint32_t caddr = ring + (uint32_t)(S * SB + p.xbytes + p.abytes);  // the constants' offsets start here
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row0 = blockIdx.x * R;
@@ -160,15 +162,15 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
   if (warp == CW) {
     if (lane != 0) return;
     if constexpr (MT > 1) {  // the prologue's constants, which depend on no preceding kernel
-      const float* src[3] = {a.inv_delta, a.rn.w_post, a.rn.w_next};
+      const float* src[3] = {pre ? nullptr : a.inv_delta, a.rn.w_post, a.rn.w_next};
       int n = 0;
 #pragma unroll
-      for (int i = 0; i < 3; ++i) n += p.coff[i] >= 0;
+      for (int i = 0; i < 3; ++i) n += src[i] && p.coff[i] >= 0;
       if (n) {
         mbar_arrive_expect_tx(smem_u32(&s_cbar), (uint32_t)(n * a.K * 4));
 #pragma unroll
         for (int i = 0; i < 3; ++i)
-          if (p.coff[i] >= 0) bulk_g2s(caddr + (uint32_t)p.coff[i], src[i], (uint32_t)(a.K * 4), smem_u32(&s_cbar));
+          if (src[i] && p.coff[i] >= 0) bulk_g2s(caddr + (uint32_t)p.coff[i], src[i], (uint32_t)(a.K * 4), smem_u32(&s_cbar));
       }
     }
     bool ok = true;
@@ -273,7 +275,8 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
       if (tid == 0) {
         mbar_arrive_expect_tx(smem_u32(&s_xbar), (uint32_t)(a.M * a.K * 2));
         for (int m = 0; m < a.M; ++m)
-          bulk_g2s(xs + (uint32_t)(m * xsb * 2), a.X + (size_t)m * a.K, (uint32_t)(a.K * 2), smem_u32(&s_xbar));
+          bulk_g2s(xs + (uint32_t)(m * xsb * 2), (pre ? a.codes : a.X) + (size_t)m * a.K, (uint32_t)(a.K * 2),
+                   smem_u32(&s_xbar));
       }
       if constexpr (!kQ) {  // bf16: zeros past K and in slots >= M
         const int t8 = (kpad - a.K) >> 3, v8 = kpad >> 3;
@@ -282,6 +285,14 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
           *reinterpret_cast<uint4*>(xsp + ((size_t)m * xsb + a.K + 8 * c) * 2) = make_uint4(0u, 0u, 0u, 0u);
         }
         for (int i = tid; i < (MT - a.M) * v8; i += CW * 32) {
+          const int m = i / v8, c = i - m * v8;
+          *reinterpret_cast<uint4*>(xsp + ((size_t)(a.M + m) * xsb + 8 * c) * 2) = make_uint4(0u, 0u, 0u, 0u);
+        }
+      }
+      if (pre) {
+        if (tid < MT) s_sx[tid] = tid < a.M ? a.s_x[tid] : 0.0f;
+        const int v8 = a.K >> 3;
+        for (int i = tid; i < (MT - a.M) * v8; i += CW * 32) {  // zeros in slots >= M
           const int m = i / v8, c = i - m * v8;
           *reinterpret_cast<uint4*>(xsp + ((size_t)(a.M + m) * xsb + 8 * c) * 2) = make_uint4(0u, 0u, 0u, 0u);
         }
@@ -512,7 +523,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
       // tokens 13.8 us, now 11.1.)
       constexpr int kRowWarps = CW >= MT ? CW / MT : 1;          // warps on one row
       constexpr int kStep = 32 * kRowWarps;
-      const ulonglong2* idl = reinterpret_cast<const ulonglong2*>(constant(0, a.inv_delta));  // 1 / delta, two pairs each
+      const ulonglong2* idl = reinterpret_cast<const ulonglong2*>(pre ? nullptr : constant(0, a.inv_delta));  // 1 / delta, two pairs each
       const f32x2 nz = f2_neg_zero();
       const int part = warp % kRowWarps, vi0 = lane + 32 * part;
       auto smooth8 = [&](const uint4& w, int vi, f32x2 (&xh)[4]) {  // x_hat of vector vi, rounded products
@@ -527,7 +538,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
         for (int e = 0; e < 4; ++e) f2_unpack(v[e], x[2 * e], x[2 * e + 1]);
       };
 #pragma unroll 1
-      for (int m = warp / kRowWarps; m < MT; m += CW / kRowWarps) {
+      for (int m = pre ? MT : warp / kRowWarps; m < MT; m += CW / kRowWarps) {
         const bool live = m < a.M;
         const uint4* src = copied ? reinterpret_cast<const uint4*>(xsp + (size_t)m * xsb * 2)
                                   : reinterpret_cast<const uint4*>(xrows + (size_t)m * xstride);
@@ -1102,7 +1113,7 @@ SmallPlan make_small_plan(int wkind, int M, int N, int K, int kind, int sm_count
   p.smem_bytes = 1024 + p.stages * p.stage_bytes + p.xbytes + p.abytes + p.rbytes + 16 * p.stages;
   // the prologue's constants: first into the partial sums' place, then past the end as far as the SM's
   // CTAs leave room
-  const bool want[3] = {mma && int8_weights, fused_norm && p.MT > 1, fused_norm && p.MT > 1};
+  const bool want[3] = {mma && int8_weights && !(wkind == SMALL_INT8 && p.MT == 16), fused_norm && p.MT > 1, fused_norm && p.MT > 1};
   int used = 0;
   for (int i = 0; i < 3; ++i) {
     p.coff[i] = -1;
@@ -1123,6 +1134,8 @@ SmallPlan make_small_plan(int wkind, int M, int N, int K, int kind, int sm_count
 w8a8_status launch_small_gemv(int wkind, const SmallArgs& a, cudaStream_t st) {
   if (a.M == 0 || a.N == 0) return W8A8_OK;
   W8A8_CHECK_ARG(a.p.ok, W8A8_ERR_SHAPE, "small GEMV: no plan for M=%d N=%d K=%d", a.M, a.N, a.K);
+  W8A8_CHECK_ARG(a.codes || wkind != SMALL_INT8 || a.p.MT < 16, W8A8_ERR_INVALID_ARG,
+                 "small GEMV: M=%d needs the activations as codes", a.M);
   void *v0, *v1;
   take_kernel_events(&v0, &v1);
   cudaEvent_t e0 = reinterpret_cast<cudaEvent_t>(v0), e1 = reinterpret_cast<cudaEvent_t>(v1);

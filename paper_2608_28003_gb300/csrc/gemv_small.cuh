@@ -75,6 +75,10 @@ struct SmallArgs {
   const float* next_inv_delta;  // [N / 2] the down projection's 1 / delta
   const float* rowmax_in;
   int rowmax_n;
+  // W8A8 at 8 / 16 token slots, nullable: the rows' codes as fp16 [M, K] and scales [M], quantised by a
+  // kernel before this one (X is then not read)
+  const uint16_t* codes;
+  const float* s_x;
 };
 
 // fused_norm: the call computes its input with a ResNorm (needs K <= 2048)

@@ -25,6 +25,9 @@ FfnWs ffn_ws(int M, int H, int F, int sms);
 // qsum (nullable): per row, sum_k |q_tk| (the tensor-core GEMM's exactness certificate)
 w8a8_status launch_quantize_rows(const uint16_t* X, int M, int K, const float* inv_delta, int8_t* xq,
                                  uint16_t* xq_f16, float* s_x, cudaStream_t st, int* qsum = nullptr);
+// fp16 codes and scales of rows whose partial maxima of |x_hat| are known: rowmax [n][stride], row t in column t
+w8a8_status launch_quantize_known_rows(const uint16_t* X, int M, int K, const float* inv_delta, const float* rowmax, int n,
+                                       int stride, uint16_t* xq_f16, float* s_x, cudaStream_t st);
 w8a8_status launch_quantize_rows_fp8(const uint16_t* X, int M, int K, const float* inv_delta, uint8_t* xq,
                                      float* s_x, cudaStream_t st);
 w8a8_status launch_act_absmax(const uint16_t* X, int T, int K, float* absmax, cudaStream_t st);

@@ -153,6 +153,55 @@ w8a8_status launch_quantize_rows(const uint16_t* X, int M, int K, const float* i
   return W8A8_OK;
 }
 
+// The same codes from row maxima that the producer of X left behind: partial maxima of |x_hat| per row,
+// [n][stride] with row t in column t (the GeGLU epilogue of the decode GEMV).  No pass over the row
+// before the codes, so a row is spread over several blocks of 1024 elements.
+__global__ void __launch_bounds__(128) quantize_known_rows_kernel(const uint16_t* __restrict__ X, int K,
+                                                                  const float* __restrict__ inv_delta,
+                                                                  const float* __restrict__ rowmax, int n, int stride,
+                                                                  uint16_t* __restrict__ xq_f16,
+                                                                  float* __restrict__ s_x) {
+  __shared__ float red[4];
+  pdl_trigger();
+  const int row = blockIdx.y, vi = blockIdx.x * 128 + threadIdx.x;
+  const bool mine = vi < (K >> 3);
+  float d[8];
+  if (mine) {
+    const float4 d0 = reinterpret_cast<const float4*>(inv_delta)[2 * vi], d1 = reinterpret_cast<const float4*>(inv_delta)[2 * vi + 1];
+    d[0] = d0.x; d[1] = d0.y; d[2] = d0.z; d[3] = d0.w; d[4] = d1.x; d[5] = d1.y; d[6] = d1.z; d[7] = d1.w;
+  }
+  pdl_wait();
+  uint4 w = make_uint4(0u, 0u, 0u, 0u);
+  if (mine) w = reinterpret_cast<const uint4*>(X + (size_t)row * K)[vi];
+  float m = 0.0f;
+  for (int i = threadIdx.x; i < n; i += 128) m = fmaxf(m, rowmax[(size_t)i * stride + row]);
+  m = warp_max(m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  m = fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
+  const float r = m > 0.0f ? __fdiv_rn(127.0f, m) : 0.0f;  // fl32(127 / m_t)
+  if (blockIdx.x == 0 && threadIdx.x == 0) s_x[row] = __fdiv_rn(m, 127.0f);
+  if (!mine) return;
+  const float x[8] = {bf16_lo(w.x), bf16_hi(w.x), bf16_lo(w.y), bf16_hi(w.y),
+                      bf16_lo(w.z), bf16_hi(w.z), bf16_lo(w.w), bf16_hi(w.w)};
+  uint32_t h[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int q0 = max(-127, min(127, __float2int_rn(__fmul_rn(__fmul_rn(x[2 * e], d[2 * e]), r))));
+    const int q1 = max(-127, min(127, __float2int_rn(__fmul_rn(__fmul_rn(x[2 * e + 1], d[2 * e + 1]), r))));
+    h[e] = f16_codes(q0, q1);
+  }
+  reinterpret_cast<uint4*>(xq_f16 + (size_t)row * K)[vi] = make_uint4(h[0], h[1], h[2], h[3]);
+}
+
+w8a8_status launch_quantize_known_rows(const uint16_t* X, int M, int K, const float* inv_delta, const float* rowmax, int n,
+                                       int stride, uint16_t* xq_f16, float* s_x, cudaStream_t st) {
+  if (M == 0) return W8A8_OK;
+  W8A8_CUDA(launch_pdl(quantize_known_rows_kernel, dim3((unsigned)((K / 8 + 127) / 128), (unsigned)M), dim3(128), 0, st, X, K,
+                       inv_delta, rowmax, n, stride, xq_f16, s_x));
+  return W8A8_OK;
+}
+
 w8a8_status launch_quantize_rows_fp8(const uint16_t* X, int M, int K, const float* inv_delta, uint8_t* xq,
                                      float* s_x, cudaStream_t st) {
   if (M == 0) return W8A8_OK;

@@ -33,3 +33,24 @@ def test_codes_match_the_standalone_quantiser(M, K, N):
     want = (s_x[:, None] * q.s_w[None, :]) * acc.float()
     assert torch.equal(y.view(torch.int16), want.to(torch.bfloat16).view(torch.int16)) or \
         torch.equal(torch.nan_to_num(y.float()), torch.nan_to_num(want.to(torch.bfloat16).float()))
+
+
+@pytest.mark.parametrize("F", [32, 4112, 6912])  # fused quantiser; known maxima: a ragged second chunk; the decoder's
+@pytest.mark.parametrize("M", [5, 8, 16])
+def test_ffn_down_equals_the_linear_on_its_input(M, F):
+    from paper_2608_28003_gb300 import build
+    build.build()
+    from paper_2608_28003_gb300 import binding as B
+    H = 1152
+    g = torch.Generator("cuda").manual_seed(F + M)
+    x = torch.randn(M, H, device="cuda", generator=g)
+    x[1, 3], x[2], x[3, 1] = float("nan"), 0.0, 1e38
+    x = x.to(torch.bfloat16)
+    wg, wu = (torch.randn(F, H, device="cuda", generator=g).to(torch.bfloat16) * 0.05 for _ in range(2))
+    wd = torch.randn(H, F, device="cuda", generator=g).to(torch.bfloat16) * 0.05
+    gu = B.prepare_gate_up(wg, wu, torch.rand(H, device="cuda", generator=g) + 0.5)
+    dn = B.prepare_weights(wd, torch.rand(F, device="cuda", generator=g) + 0.5)
+    f = B.FfnWeights(H, F, gu, dn, B.interleave_gate_up(wg, wu), wd)
+    y, h = B.ffn_block(f, B.W8A8_PREC_W8A8, x, want_h=True)
+    want = B.linear(f.down, h)
+    assert torch.equal(y.view(torch.int16), want.view(torch.int16))
