@@ -116,8 +116,6 @@ struct RowMax {
   int n;                        // down: gate/up's CTA count
 };
 
-constexpr int kSeparateK1MinK = 4096;  // at 5-8 tokens; between the two measured lengths 1152 and 6912
-
 static bool small_gemv(bool int8, const void* W, const float* inv_delta, const float* s_w, const uint16_t* X, int M,
                        int N, int K, const float* bias, int kind, uint16_t* Y, const w8a8_debug* dbg, void* ws,
                        const ResNorm* rn, int sms, cudaStream_t st, w8a8_status* status, const RowMax* rm = nullptr,
@@ -126,13 +124,9 @@ static bool small_gemv(bool int8, const void* W, const float* inv_delta, const f
   SmallArgs a{};
   a.p = make_small_plan(int8, M, N, K, kind, sms, rn != nullptr);
   if (!a.p.ok) return false;
-  // Every CTA of this kernel needs all the codes.  Where its own pass over the rows takes longer than a
-  // launch of the quantiser (one block per row, or several where the row maxima are known), that launch
-  // writes them to `codes` and `s_x`, unless the producer of X has already: W8A8 1152 -> 6912 at 16 tokens
-  // 11.0 -> 9.5 us, 6912 -> 1152 at 8 tokens 11.4 -> 9.0, the FFN block at 8 tokens 20.2 -> 18.9.  At 5-8
-  // tokens and K = 1152 the pass takes under 2 us, less than a launch (1152 -> 6912: 7.6 us with it).
-  const bool known = rm && rm->in, long_k = K >= kSeparateK1MinK;
-  if (int8 && a.p.MT >= 8 && codes && !rn && (a.p.MT == 16 || long_k)) {
+  // The quantiser's own launch writes `codes` and `s_x`, unless the producer of X has written its codes.
+  const bool known = rm && rm->in;
+  if (int8 && codes && !rn && separate_k1(a.p, K)) {
     if (pre && pre->codes16 && !dbg) {
       a.codes = pre->codes16;
       a.s_x = pre->s_x;

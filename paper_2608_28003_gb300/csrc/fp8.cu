@@ -5,8 +5,9 @@
 // the code products in fp32 (not exact: a sum of e4m3 products needs up to 49 bits) and the
 // epilogue dequantises y = fl32(fl32(s_x s_w) * acc) (+ bias), the order of Eq. gemm-final.
 //
-// Routing: 1-8 tokens run the row-owning decode GEMV on its tensor-core path (e4m3 weights and
-// codes widened to fp16, K1 fused); more tokens run the per-token quantiser, then the tcgen05 GEMM
+// Routing: 1-16 tokens run the row-owning decode GEMV on its tensor-core path where it takes the shape
+// (e4m3 weights and codes widened to fp16; K1 fused, or a launch before it at 9-16 tokens or a long K);
+// other calls run the per-token quantiser, then the tcgen05 GEMM
 // with kind::f8f6f4 on the one-byte codes (no wider copy of the weights exists or is needed).
 #include "common.cuh"
 #include "gemm_tc.cuh"
@@ -37,7 +38,16 @@ w8a8_status run_fp8_linear(const w8a8_fp8_weight* w, const uint16_t* X, int M, c
   const int N = w->n, K = w->k;
   SmallArgs s{};
   s.p = make_small_plan(SMALL_FP8, M, N, K, kind, sms, false);
+  const LinearWs L = linear_ws(M, N, K, true, sms);
+  char* codes = scratch + (L.xf16 - W8A8_WS_RESERVED);
+  float* s_x = reinterpret_cast<float*>(scratch + (L.sx - W8A8_WS_RESERVED));
   if (s.p.ok) {
+    if (separate_k1(s.p, K)) {
+      W8A8_TRY(launch_quantize_rows_fp8(X, M, K, w->inv_delta, xq_dbg, s_x, st, reinterpret_cast<uint16_t*>(codes)));
+      if (s_x_dbg) W8A8_CUDA(cudaMemcpyAsync(s_x_dbg, s_x, sizeof(float) * M, cudaMemcpyDeviceToDevice, st));
+      s.codes = reinterpret_cast<uint16_t*>(codes);
+      s.s_x = s_x;
+    }
     s.W = w->wq;
     s.X = X;
     s.M = M;
@@ -55,10 +65,7 @@ w8a8_status run_fp8_linear(const w8a8_fp8_weight* w, const uint16_t* X, int M, c
   }
   W8A8_CHECK_ARG(tc_gemm_supported(M, N, K, kind, false, 0), W8A8_ERR_SHAPE,
                  "fp8 linear: no kernel takes M=%d N=%d K=%d", M, N, K);
-  const LinearWs L = linear_ws(M, N, K, true, sms);
-  uint8_t* codes = reinterpret_cast<uint8_t*>(scratch + (L.xf16 - W8A8_WS_RESERVED));
-  float* s_x = reinterpret_cast<float*>(scratch + (L.sx - W8A8_WS_RESERVED));
-  W8A8_TRY(launch_quantize_rows_fp8(X, M, K, w->inv_delta, codes, s_x, st));
+  W8A8_TRY(launch_quantize_rows_fp8(X, M, K, w->inv_delta, reinterpret_cast<uint8_t*>(codes), s_x, st));
   if (xq_dbg) W8A8_CUDA(cudaMemcpyAsync(xq_dbg, codes, (size_t)M * K, cudaMemcpyDeviceToDevice, st));
   if (s_x_dbg) W8A8_CUDA(cudaMemcpyAsync(s_x_dbg, s_x, sizeof(float) * M, cudaMemcpyDeviceToDevice, st));
   TcArgs a{};

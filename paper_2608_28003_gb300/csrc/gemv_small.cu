@@ -130,12 +130,14 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
   uint64_t* full =
       reinterpret_cast<uint64_t*>(smem_raw + (ring - raw) + (size_t)S * SB + p.xbytes + p.abytes + p.rbytes);
   uint64_t* empty = full + S;
-  const bool pre = kInt8 && (MT == 16 || (kMma && a.codes));  // the activations come as codes: no quantiser here
+  const bool pre = kQ && (MT == 16 || (kMma && a.codes));  // the activations come as codes: no quantiser here
   const uint32_t caddr = ring + (uint32_t)(S * SB + p.xbytes + p.abytes);  // the constants' offsets start here
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row0 = blockIdx.x * R;
-  // the fused residual norm runs at 1-8 token slots on 8 consumer warps (no other call is planned with it)
-  constexpr bool kRn = CW == kCW && MT <= 8 && !kFp8;
+  // The fused residual norm runs at 1-8 token slots on 8 consumer warps; no other call is planned with it,
+  // and none in FP8, where its code stays at 1-2 slots all the same: without it the compiler holds fewer
+  // of the quantiser's operands in registers (6912 -> 1152 at 1 token 9.1 us against 7.4).
+  constexpr bool kRn = CW == kCW && MT <= 8 && (!kFp8 || MT <= 2);
   if constexpr (!kRn) {
     if (a.has_rn) {
       if (threadIdx.x == 0) atomicOr(a.err, DEVERR_CONSUMER_WAIT);
@@ -458,11 +460,19 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
         const bool live = m < a.M;
         if (live) {
           const uint4* src = reinterpret_cast<const uint4*>(xrows + (size_t)m * xstride);
+          // 1-2 slots: the row's loads together ahead of their use (W8A8 6912 -> 1152 at 1 token 4.8 -> 4.4
+          // us, a decode step 577 -> 573); at 4 slots that made short rows slower (1152 -> 1536 5.1 -> 5.5)
+          uint4 xw[4];
+          if constexpr (MT <= 2) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+              if (tid + v * CW * 32 < nvec) xw[v] = src[tid + v * CW * 32];
+          }
 #pragma unroll
           for (int v = 0; v < 4; ++v) {
             const int vi = tid + v * CW * 32;
             if (vi < nvec) {
-              const uint4 w = src[vi];
+              const uint4 w = MT <= 2 ? xw[v] : src[vi];
               const float4 d0 = idr[v][0], d1 = idr[v][1];
               xh[v][0] = __fmul_rn(bf16_lo(w.x), d0.x);
               xh[v][1] = __fmul_rn(bf16_hi(w.x), d0.y);
@@ -1113,7 +1123,7 @@ SmallPlan make_small_plan(int wkind, int M, int N, int K, int kind, int sm_count
   p.smem_bytes = 1024 + p.stages * p.stage_bytes + p.xbytes + p.abytes + p.rbytes + 16 * p.stages;
   // the prologue's constants: first into the partial sums' place, then past the end as far as the SM's
   // CTAs leave room
-  const bool want[3] = {mma && int8_weights && !(wkind == SMALL_INT8 && p.MT == 16), fused_norm && p.MT > 1, fused_norm && p.MT > 1};
+  const bool want[3] = {mma && int8_weights && p.MT < 16, fused_norm && p.MT > 1, fused_norm && p.MT > 1};
   int used = 0;
   for (int i = 0; i < 3; ++i) {
     p.coff[i] = -1;
@@ -1134,7 +1144,7 @@ SmallPlan make_small_plan(int wkind, int M, int N, int K, int kind, int sm_count
 w8a8_status launch_small_gemv(int wkind, const SmallArgs& a, cudaStream_t st) {
   if (a.M == 0 || a.N == 0) return W8A8_OK;
   W8A8_CHECK_ARG(a.p.ok, W8A8_ERR_SHAPE, "small GEMV: no plan for M=%d N=%d K=%d", a.M, a.N, a.K);
-  W8A8_CHECK_ARG(a.codes || wkind != SMALL_INT8 || a.p.MT < 16, W8A8_ERR_INVALID_ARG,
+  W8A8_CHECK_ARG(a.codes || wkind == SMALL_BF16 || a.p.MT < 16, W8A8_ERR_INVALID_ARG,
                  "small GEMV: M=%d needs the activations as codes", a.M);
   void *v0, *v1;
   take_kernel_events(&v0, &v1);

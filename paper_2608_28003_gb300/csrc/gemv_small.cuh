@@ -75,14 +75,22 @@ struct SmallArgs {
   const float* next_inv_delta;  // [N / 2] the down projection's 1 / delta
   const float* rowmax_in;
   int rowmax_n;
-  // W8A8 at 8 / 16 token slots, nullable: the rows' codes as fp16 [M, K] and scales [M], quantised by a
-  // kernel before this one (X is then not read)
+  // W8A8 and FP8 at 8 / 16 token slots: the rows' codes as fp16 [M, K] and scales [M], quantised by a
+  // kernel before this one (X is then not read); null at 8 slots: quantised here
   const uint16_t* codes;
   const float* s_x;
 };
 
 // fused_norm: the call computes its input with a ResNorm (needs K <= 2048)
 SmallPlan make_small_plan(int wkind, int M, int N, int K, int kind, int sm_count, bool fused_norm = false);
+
+// Whether the codes of a W8A8 or FP8 call (without a fused residual norm) come from a launch before the
+// GEMV.  Every CTA of the GEMV needs all of them, so where its own pass over the rows takes longer than a
+// launch of the quantiser, that is faster: W8A8 1152 -> 6912 at 16 tokens 11.0 -> 9.5 us, 6912 -> 1152 at 8
+// tokens 11.4 -> 9.0, the FFN block at 8 tokens 20.2 -> 18.9.  At 5-8 tokens and K = 1152 the pass takes
+// under 2 us, less than a launch (1152 -> 6912: 7.6 us with it).  The line lies between those two lengths.
+constexpr int kSeparateK1MinK = 4096;
+inline bool separate_k1(const SmallPlan& p, int K) { return p.MT == 16 || (p.MT == 8 && K >= kSeparateK1MinK); }
 w8a8_status launch_small_gemv(int wkind, const SmallArgs& a, cudaStream_t st);
 
 }  // namespace w8a8

@@ -29,12 +29,13 @@ w8a8_status launch_quantize_rows(const uint16_t* X, int M, int K, const float* i
 w8a8_status launch_quantize_known_rows(const uint16_t* X, int M, int K, const float* inv_delta, const float* rowmax, int n,
                                        int stride, uint16_t* xq_f16, float* s_x, cudaStream_t st);
 w8a8_status launch_quantize_rows_fp8(const uint16_t* X, int M, int K, const float* inv_delta, uint8_t* xq,
-                                     float* s_x, cudaStream_t st);
+                                     float* s_x, cudaStream_t st, uint16_t* xq_f16 = nullptr);
 w8a8_status launch_act_absmax(const uint16_t* X, int T, int K, float* absmax, cudaStream_t st);
 
 // The per-token quantiser's outputs for X computed by the kernel that produced X (the decoder's
 // norm kernels): fp16 codes [M, K], s_x [M] and the rows' sums of |codes| [M] (nullable).  A W8A8
-// linear that runs the tensor-core GEMM then launches no quantiser of its own; other routes
+// linear that runs the tensor-core GEMM or, at 9-16 tokens, the decode GEMV then launches no quantiser
+// of its own; other routes
 // quantise X themselves and ignore them.
 struct PreCodes {
   const uint16_t* codes16;

@@ -83,11 +83,14 @@ __global__ void __launch_bounds__(256) quantize_rows_kernel(const uint16_t* __re
 
   int qs = 0;  // sum_k |q_tk| of this thread's codes (the GEMM's exactness certificate)
   auto emit = [&](int vi, const float (&v8)[8]) {
-    if constexpr (kFp8) {  // e4m3 codes (xq receives the bytes)
+    if constexpr (kFp8) {  // e4m3 codes: the bytes in xq, their fp16 values in xq_f16
       uint32_t c[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) c[e] = e4m3x2_of(__fmul_rn(v8[2 * e], r), __fmul_rn(v8[2 * e + 1], r));
-      reinterpret_cast<uint2*>(xq + (size_t)row * K)[vi] = make_uint2(c[0] | (c[1] << 16), c[2] | (c[3] << 16));
+      if (xq) reinterpret_cast<uint2*>(xq + (size_t)row * K)[vi] = make_uint2(c[0] | (c[1] << 16), c[2] | (c[3] << 16));
+      if (xq_f16)
+        reinterpret_cast<uint4*>(xq_f16 + (size_t)row * K)[vi] =
+            make_uint4(e4m3x2_to_f16x2(c[0]), e4m3x2_to_f16x2(c[1]), e4m3x2_to_f16x2(c[2]), e4m3x2_to_f16x2(c[3]));
     } else {
       int q[8];
 #pragma unroll
@@ -203,12 +206,12 @@ w8a8_status launch_quantize_known_rows(const uint16_t* X, int M, int K, const fl
 }
 
 w8a8_status launch_quantize_rows_fp8(const uint16_t* X, int M, int K, const float* inv_delta, uint8_t* xq,
-                                     float* s_x, cudaStream_t st) {
+                                     float* s_x, cudaStream_t st, uint16_t* xq_f16) {
   if (M == 0) return W8A8_OK;
   const int nvec = K / 8;
   const int threads = nvec <= 4 * 128 ? 128 : 256;
   W8A8_CUDA(launch_pdl(quantize_rows_kernel<4, true>, dim3(M), dim3(threads), 0, st, X, K, inv_delta,
-                       reinterpret_cast<int8_t*>(xq), static_cast<uint16_t*>(nullptr), s_x, static_cast<int*>(nullptr)));
+                       reinterpret_cast<int8_t*>(xq), xq_f16, s_x, static_cast<int*>(nullptr)));
   return W8A8_OK;
 }
 
@@ -559,5 +562,5 @@ extern "C" w8a8_status w8a8_fp8_quantize_activations(const uint16_t* X, int M, i
                  "w8a8_fp8_quantize_activations: pointers must be 16-byte aligned");
   w8a8_status s = check_device();
   if (s != W8A8_OK) return s;
-  return launch_quantize_rows_fp8(X, M, K, inv_delta, xq, s_x, as_stream(stream));
+  return launch_quantize_rows_fp8(X, M, K, inv_delta, xq, s_x, as_stream(stream), nullptr);
 }
