@@ -16,10 +16,10 @@ struct StreamPlan {
   int TOK;      // tokens per group = 8 * NB
   int Z;        // token groups
   int G;        // 128-row weight groups
-  int KC;       // k elements per pipeline stage
+  int KC;       // k elements per unit
   int C;        // k chunks per row group
   int P;        // CTAs (persistent, one per SM)
-  int stages;   // pipeline depth
+  int stages;   // units that fit in the ring's room (the dp4a path's pipeline depth)
   int stage_bytes;
   int slots;    // ring slots of the streaming kernel: one weight box each, with its token boxes unless resident
   int xres;     // bytes of the token rows when they stay in shared memory (one token group), else 0
