@@ -13,7 +13,8 @@
  *     weight [N, K] has one row per output channel i and one column per input channel j
  *     (the paper's W_{i,j}).
  *   - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).  Compute
- *     calls are asynchronous on it.  Errors found on the host (arguments, shapes,
+ *     calls are asynchronous on it and run in stream order: every argument, weights and scales
+ *     included, may be the result of earlier work on the stream.  Errors found on the host (arguments, shapes,
  *     alignment) are reported before anything is launched.  Errors of a launch are
  *     reported as W8A8_ERR_CUDA.
  *   - Alignment: every tensor pointer must be 16-byte aligned, and every K (input channels)

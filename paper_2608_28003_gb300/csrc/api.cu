@@ -93,13 +93,13 @@ static w8a8_status check_ws(const char* who, void* ws, size_t have, size_t need)
 // Per-token quantiser for a W8A8 GEMM plan: INT8 codes for the dp4a GEMV, fp16 codes for the MMA
 // kernel, written to `codes` (workspace); `xq_dbg` (nullable) also receives the INT8 codes.
 static w8a8_status quantize_for(const StreamPlan& p, const uint16_t* X, int M, int K, const float* inv_delta,
-                                void* codes, int8_t* xq_dbg, float* s_x, cudaStream_t st) {
+                                void* codes, int8_t* xq_dbg, float* s_x, cudaStream_t st, bool settled) {
   if (p.dp4a) {
-    W8A8_TRY(launch_quantize_rows(X, M, K, inv_delta, reinterpret_cast<int8_t*>(codes), nullptr, s_x, st));
+    W8A8_TRY(launch_quantize_rows(X, M, K, inv_delta, reinterpret_cast<int8_t*>(codes), nullptr, s_x, st, settled));
     if (xq_dbg) W8A8_CUDA(cudaMemcpyAsync(xq_dbg, codes, (size_t)M * K, cudaMemcpyDeviceToDevice, st));
     return W8A8_OK;
   }
-  return launch_quantize_rows(X, M, K, inv_delta, xq_dbg, reinterpret_cast<uint16_t*>(codes), s_x, st);
+  return launch_quantize_rows(X, M, K, inv_delta, xq_dbg, reinterpret_cast<uint16_t*>(codes), s_x, st, settled);
 }
 
 static unsigned int* err_word(void* ws) {
@@ -118,7 +118,7 @@ struct RowMax {
 
 static bool small_gemv(bool int8, const void* W, const float* inv_delta, const float* s_w, const uint16_t* X, int M,
                        int N, int K, const float* bias, int kind, uint16_t* Y, const w8a8_debug* dbg, void* ws,
-                       const ResNorm* rn, int sms, cudaStream_t st, w8a8_status* status, const RowMax* rm = nullptr,
+                       const ResNorm* rn, int sms, cudaStream_t st, bool settled, w8a8_status* status, const RowMax* rm = nullptr,
                        const PreCodes* pre = nullptr, uint16_t* codes = nullptr, float* s_x = nullptr) {
   if (kind != EPI_BF16 && kind != EPI_GEGLU) return false;
   SmallArgs a{};
@@ -134,7 +134,7 @@ static bool small_gemv(bool int8, const void* W, const float* inv_delta, const f
       if (known)
         *status = launch_quantize_known_rows(X, M, K, inv_delta, rm->in, rm->n, a.p.MT, codes, s_x, st);
       else
-        *status = launch_quantize_rows(X, M, K, inv_delta, dbg ? dbg->xq : nullptr, codes, s_x, st);
+        *status = launch_quantize_rows(X, M, K, inv_delta, dbg ? dbg->xq : nullptr, codes, s_x, st, settled);
       if (*status == W8A8_OK && dbg && dbg->s_x &&
           cudaMemcpyAsync(dbg->s_x, s_x, sizeof(float) * M, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
         *status = W8A8_ERR_CUDA;
@@ -167,6 +167,7 @@ static bool small_gemv(bool int8, const void* W, const float* inv_delta, const f
   a.s_x_dbg = dbg ? dbg->s_x : nullptr;
   a.acc_dbg = dbg ? dbg->acc : nullptr;
   a.err = err_word(ws);
+  a.settled = settled || a.codes;  // after the quantiser's launch
   *status = launch_small_gemv(int8, a, st);
   return true;
 }
@@ -194,7 +195,7 @@ static bool head_bf16_on_tc(int M, int N, int K) {
 static bool tc_path(bool int8, const void* W16, const uint16_t* X, int M, int N, int K, const float* bias, int kind,
                     const float* inv_delta, const float* s_w, uint16_t* Y, float* logits, int32_t* top1,
                     const w8a8_debug* dbg, void* ws, void* codes, float* s_x, void* part, cudaStream_t st,
-                    w8a8_status* status, const PreCodes* pre = nullptr) {
+                    bool settled, w8a8_status* status, const PreCodes* pre = nullptr) {
   if (M < (N <= kTcNarrowMaxN ? kTcMinTokensNarrow : int8 ? kTcMinTokensWideInt8 : kTcMinTokensWideBf16) || !W16 ||
       !tc_gemm_supported(M, N, K, kind, top1 != nullptr, max_top_keys()))
     return false;
@@ -207,7 +208,7 @@ static bool tc_path(bool int8, const void* W16, const uint16_t* X, int M, int N,
   } else if (int8) {
     int* qsum = reinterpret_cast<int*>(s_x + M);  // beside s_x in the workspace
     w8a8_status q = launch_quantize_rows(X, M, K, inv_delta, dbg ? dbg->xq : nullptr,
-                                         reinterpret_cast<uint16_t*>(codes), s_x, st, qsum);
+                                         reinterpret_cast<uint16_t*>(codes), s_x, st, settled, qsum);
     if (q == W8A8_OK && dbg && dbg->s_x)
       q = cudaMemcpyAsync(dbg->s_x, s_x, sizeof(float) * M, cudaMemcpyDeviceToDevice, st) == cudaSuccess
               ? W8A8_OK
@@ -240,6 +241,7 @@ static bool tc_path(bool int8, const void* W16, const uint16_t* X, int M, int N,
   a.err = r.err;
   a.partials = part;
   a.tile_counters = r.tile_counters;
+  a.settled = settled || int8;  // W8A8: after the quantiser
   *status = launch_tc_gemm(int8 ? TC_I8 : TC_BF16, a, st);
   return true;
 }
@@ -247,7 +249,7 @@ static bool tc_path(bool int8, const void* W16, const uint16_t* X, int M, int N,
 // One W8A8 linear: K1 then the streaming GEMM.  s_x and the codes live in the workspace.
 w8a8_status run_w8a8_linear(const w8a8_qweight* w, const uint16_t* X, int M, const float* bias, int kind,
                                    uint16_t* Y, float* logits, int32_t* top1, const w8a8_debug* dbg, void* ws,
-                                   int sms, cudaStream_t st, const ResNorm* rn, const PreCodes* pre) {
+                                   int sms, cudaStream_t st, bool settled, const ResNorm* rn, const PreCodes* pre) {
   const int N = w->n, K = w->k;
   w8a8_status small_status = W8A8_OK;
   LinearWs L = linear_ws(M, N, K, true, sms);
@@ -255,16 +257,16 @@ w8a8_status run_w8a8_linear(const w8a8_qweight* w, const uint16_t* X, int M, con
   void* codes = base + L.xf16;
   float* s_x = reinterpret_cast<float*>(base + L.sx);
   if (!logits && !top1 &&
-      small_gemv(true, w->wq, w->inv_delta, w->s_w, X, M, N, K, bias, kind, Y, dbg, ws, rn, sms, st, &small_status, nullptr,
-                 pre, reinterpret_cast<uint16_t*>(codes), s_x))
+      small_gemv(true, w->wq, w->inv_delta, w->s_w, X, M, N, K, bias, kind, Y, dbg, ws, rn, sms, st, settled, &small_status,
+                 nullptr, pre, reinterpret_cast<uint16_t*>(codes), s_x))
     return small_status;
   W8A8_CHECK_ARG(!rn, W8A8_ERR_SHAPE, "fused residual norm: the decode GEMV does not take M=%d N=%d K=%d", M, N, K);
   if (tc_path(true, w->wq_f16, X, M, N, K, bias, kind, w->inv_delta, w->s_w, Y, logits, top1, dbg, ws, codes, s_x,
-              base + L.part, st, &small_status, pre))
+              base + L.part, st, settled, &small_status, pre))
     return small_status;
   StreamArgs a{};
   a.p = make_stream_plan(true, M, N, K, sms);
-  W8A8_TRY(quantize_for(a.p, X, M, K, w->inv_delta, codes, dbg ? dbg->xq : nullptr, s_x, st));
+  W8A8_TRY(quantize_for(a.p, X, M, K, w->inv_delta, codes, dbg ? dbg->xq : nullptr, s_x, st, settled));
   if (dbg && dbg->s_x) W8A8_CUDA(cudaMemcpyAsync(dbg->s_x, s_x, sizeof(float) * M, cudaMemcpyDeviceToDevice, st));
   a.W = w->wq;
   a.X = codes;
@@ -281,20 +283,21 @@ w8a8_status run_w8a8_linear(const w8a8_qweight* w, const uint16_t* X, int M, con
   a.acc_dbg = dbg ? dbg->acc : nullptr;
   a.partials = base + L.part;
   attach_reserved(a, ws);
+  a.settled = 1;  // after the quantiser
   return launch_stream_gemm(true, a, st);
 }
 
 w8a8_status run_bf16_linear(const uint16_t* W, int N, int K, const uint16_t* X, int M, const float* bias,
                                    int kind, uint16_t* Y, float* logits, int32_t* top1, void* ws, int sms,
-                                   cudaStream_t st, const ResNorm* rn) {
+                                   cudaStream_t st, bool settled, const ResNorm* rn) {
   w8a8_status small_status = W8A8_OK;
   if (!logits && !top1 &&
-      small_gemv(false, W, nullptr, nullptr, X, M, N, K, bias, kind, Y, nullptr, ws, rn, sms, st, &small_status))
+      small_gemv(false, W, nullptr, nullptr, X, M, N, K, bias, kind, Y, nullptr, ws, rn, sms, st, settled, &small_status))
     return small_status;
   W8A8_CHECK_ARG(!rn, W8A8_ERR_SHAPE, "fused residual norm: the decode GEMV does not take M=%d N=%d K=%d", M, N, K);
   LinearWs L = linear_ws(M, N, K, false, sms);
   if (tc_path(false, W, X, M, N, K, bias, kind, nullptr, nullptr, Y, logits, top1, nullptr, ws, nullptr, nullptr,
-              reinterpret_cast<char*>(ws) + L.part, st, &small_status))
+              reinterpret_cast<char*>(ws) + L.part, st, settled, &small_status))
     return small_status;
   StreamArgs a{};
   a.W = W;
@@ -310,6 +313,7 @@ w8a8_status run_bf16_linear(const uint16_t* W, int N, int K, const uint16_t* X, 
   a.top1 = top1;
   a.partials = reinterpret_cast<char*>(ws) + L.part;
   attach_reserved(a, ws);
+  a.settled = settled;
   return launch_stream_gemm(false, a, st);
 }
 
@@ -321,7 +325,7 @@ w8a8_status linear_on_scratch(const w8a8_qweight* w, const uint16_t* X, int M, c
   DevInfo d;
   W8A8_TRY(dev_info(&d));
   W8A8_TRY(check_ws("w8a8_linear_noalloc", scratch, scratch_bytes, linear_ws(M, w->n, w->k, true, d.sms).total));
-  return run_w8a8_linear(w, X, M, bias, EPI_BF16, Y, nullptr, nullptr, nullptr, scratch, d.sms, st);
+  return run_w8a8_linear(w, X, M, bias, EPI_BF16, Y, nullptr, nullptr, nullptr, scratch, d.sms, st, false);
 }
 
 w8a8_status check_linear_args(const char* who, const w8a8_qweight* w, const uint16_t* X, int M, const float* bias,
@@ -427,7 +431,7 @@ extern "C" w8a8_status w8a8_linear(const w8a8_qweight* w, const uint16_t* X, int
   DevInfo d;
   W8A8_TRY(dev_info(&d));
   W8A8_TRY(check_ws("w8a8_linear", workspace, ws_bytes, linear_ws(M, w->n, w->k, true, d.sms).total));
-  return run_w8a8_linear(w, X, M, bias, EPI_BF16, Y, nullptr, nullptr, dbg, workspace, d.sms, as_stream(stream));
+  return run_w8a8_linear(w, X, M, bias, EPI_BF16, Y, nullptr, nullptr, dbg, workspace, d.sms, as_stream(stream), false);
 }
 
 extern "C" w8a8_status w8a8_linear_bf16_workspace_size(int M, int N, int K, size_t* bytes) {
@@ -448,7 +452,8 @@ extern "C" w8a8_status w8a8_linear_bf16(const uint16_t* W, int N, int K, const u
   DevInfo d;
   W8A8_TRY(dev_info(&d));
   W8A8_TRY(check_ws("w8a8_linear_bf16", workspace, ws_bytes, linear_ws(M, N, K, false, d.sms).total));
-  return run_bf16_linear(W, N, K, X, M, bias, EPI_BF16, Y, nullptr, nullptr, workspace, d.sms, as_stream(stream));
+  return run_bf16_linear(W, N, K, X, M, bias, EPI_BF16, Y, nullptr, nullptr, workspace, d.sms, as_stream(stream),
+                         false);
 }
 
 // ------------------------------------------------------------------------------- FFN
@@ -474,7 +479,8 @@ FfnWs ffn_ws(int M, int H, int F, int sms) {
 }
 
 w8a8_status run_ffn(const w8a8_ffn_weights* f, int precision, const uint16_t* X, int M, uint16_t* Y, uint16_t* h_dbg,
-                    void* workspace, int sms, cudaStream_t st, const ResNorm* rn_gate_up, const PreCodes* pre_gate_up) {
+                    void* workspace, int sms, cudaStream_t st, bool settled, const ResNorm* rn_gate_up,
+                    const PreCodes* pre_gate_up) {
   const int H = f->hidden, F = f->inter;
   const FfnWs L = ffn_ws(M, H, F, sms);
   char* base = reinterpret_cast<char*>(workspace);
@@ -493,7 +499,7 @@ w8a8_status run_ffn(const w8a8_ffn_weights* f, int precision, const uint16_t* X,
     const LinearWs lg = linear_ws(M, 2 * F, H, true, sms), ld = linear_ws(M, H, F, true, sms);
     char *gu = base + L.gu - W8A8_WS_RESERVED, *dn = base + L.dn - W8A8_WS_RESERVED;  // + a LinearWs offset
     if (small_gemv(true, f->gate_up.wq, f->gate_up.inv_delta, f->gate_up.s_w, X, M, 2 * F, H, nullptr, EPI_GEGLU, h,
-                   nullptr, workspace, rn_gate_up, sms, st, &ss, handoff ? &rm_gu : nullptr, pre_gate_up,
+                   nullptr, workspace, rn_gate_up, sms, st, settled, &ss, handoff ? &rm_gu : nullptr, pre_gate_up,
                    reinterpret_cast<uint16_t*>(gu + lg.xf16), reinterpret_cast<float*>(gu + lg.sx))) {
       W8A8_TRY(ss);
     } else if (rn_gate_up) {
@@ -502,7 +508,7 @@ w8a8_status run_ffn(const w8a8_ffn_weights* f, int precision, const uint16_t* X,
                        f->gate_up.s_w, h, nullptr, nullptr, nullptr, workspace,
                        base + L.gu + (lg.xf16 - W8A8_WS_RESERVED),
                        reinterpret_cast<float*>(base + L.gu + (lg.sx - W8A8_WS_RESERVED)),
-                       base + L.gu + (lg.part - W8A8_WS_RESERVED), st, &ss,
+                       base + L.gu + (lg.part - W8A8_WS_RESERVED), st, settled, &ss,
                        pre_gate_up)) {
       W8A8_TRY(ss);
     } else {
@@ -511,7 +517,7 @@ w8a8_status run_ffn(const w8a8_ffn_weights* f, int precision, const uint16_t* X,
       float* s_x = reinterpret_cast<float*>(base + L.gu + (A.sx - W8A8_WS_RESERVED));
       StreamArgs a{};
       a.p = make_stream_plan(true, M, 2 * F, H, sms);
-      W8A8_TRY(quantize_for(a.p, X, M, H, f->gate_up.inv_delta, codes, nullptr, s_x, st));
+      W8A8_TRY(quantize_for(a.p, X, M, H, f->gate_up.inv_delta, codes, nullptr, s_x, st, settled));
       a.W = f->gate_up.wq;
       a.X = codes;
       a.M = M;
@@ -523,17 +529,18 @@ w8a8_status run_ffn(const w8a8_ffn_weights* f, int precision, const uint16_t* X,
       a.y = h;
       a.partials = base + L.gu + (A.part - W8A8_WS_RESERVED);
       attach_reserved(a, workspace);
+      a.settled = 1;  // after the quantiser
       W8A8_TRY(launch_stream_gemm(true, a, st));
     }
     if (small_gemv(true, f->down.wq, f->down.inv_delta, f->down.s_w, h, M, H, F, nullptr, EPI_BF16, Y, nullptr,
-                   workspace, nullptr, sms, st, &ss, handoff ? &rm_dn : nullptr, nullptr,
+                   workspace, nullptr, sms, st, true, &ss, handoff ? &rm_dn : nullptr, nullptr,
                    reinterpret_cast<uint16_t*>(dn + ld.xf16), reinterpret_cast<float*>(dn + ld.sx))) {
       W8A8_TRY(ss);
     } else if (tc_path(true, f->down.wq_f16, h, M, H, F, nullptr, EPI_BF16, f->down.inv_delta, f->down.s_w, Y,
                        nullptr, nullptr, nullptr, workspace,
                        base + L.dn + (ld.xf16 - W8A8_WS_RESERVED),
                        reinterpret_cast<float*>(base + L.dn + (ld.sx - W8A8_WS_RESERVED)),
-                       base + L.dn + (ld.part - W8A8_WS_RESERVED), st, &ss)) {
+                       base + L.dn + (ld.part - W8A8_WS_RESERVED), st, true, &ss)) {
       W8A8_TRY(ss);
     } else {
       const LinearWs B = linear_ws(M, H, F, true, sms);
@@ -541,7 +548,7 @@ w8a8_status run_ffn(const w8a8_ffn_weights* f, int precision, const uint16_t* X,
       float* s_x = reinterpret_cast<float*>(base + L.dn + (B.sx - W8A8_WS_RESERVED));
       StreamArgs a{};
       a.p = make_stream_plan(true, M, H, F, sms);
-      W8A8_TRY(quantize_for(a.p, h, M, F, f->down.inv_delta, codes, nullptr, s_x, st));
+      W8A8_TRY(quantize_for(a.p, h, M, F, f->down.inv_delta, codes, nullptr, s_x, st, true));
       a.W = f->down.wq;
       a.X = codes;
       a.M = M;
@@ -553,18 +560,20 @@ w8a8_status run_ffn(const w8a8_ffn_weights* f, int precision, const uint16_t* X,
       a.y = Y;
       a.partials = base + L.dn + (B.part - W8A8_WS_RESERVED);
       attach_reserved(a, workspace);
+      a.settled = 1;  // after the quantiser
       W8A8_TRY(launch_stream_gemm(true, a, st));
     }
   } else {
     w8a8_status ss = W8A8_OK;
     if (small_gemv(false, f->gate_up_bf16, nullptr, nullptr, X, M, 2 * F, H, nullptr, EPI_GEGLU, h, nullptr,
-                   workspace, rn_gate_up, sms, st, &ss)) {
+                   workspace, rn_gate_up, sms, st, settled, &ss)) {
       W8A8_TRY(ss);
     } else if (rn_gate_up) {
       W8A8_CHECK_ARG(false, W8A8_ERR_SHAPE, "fused residual norm: the decode GEMV does not take gate/up at M=%d", M);
     } else if (tc_path(false, f->gate_up_bf16, X, M, 2 * F, H, nullptr, EPI_GEGLU, nullptr, nullptr, h, nullptr,
                        nullptr, nullptr, workspace, nullptr, nullptr,
-                       base + L.gu + (linear_ws(M, 2 * F, H, false, sms).part - W8A8_WS_RESERVED), st, &ss)) {
+                       base + L.gu + (linear_ws(M, 2 * F, H, false, sms).part - W8A8_WS_RESERVED), st, settled,
+                       &ss)) {
       W8A8_TRY(ss);
     } else {
       const LinearWs A = linear_ws(M, 2 * F, H, false, sms);
@@ -579,14 +588,15 @@ w8a8_status run_ffn(const w8a8_ffn_weights* f, int precision, const uint16_t* X,
       a.y = h;
       a.partials = base + L.gu + (A.part - W8A8_WS_RESERVED);
       attach_reserved(a, workspace);
+      a.settled = settled;
       W8A8_TRY(launch_stream_gemm(false, a, st));
     }
     if (small_gemv(false, f->down_bf16, nullptr, nullptr, h, M, H, F, nullptr, EPI_BF16, Y, nullptr, workspace,
-                   nullptr, sms, st, &ss)) {
+                   nullptr, sms, st, true, &ss)) {
       W8A8_TRY(ss);
     } else if (tc_path(false, f->down_bf16, h, M, H, F, nullptr, EPI_BF16, nullptr, nullptr, Y, nullptr, nullptr,
                        nullptr, workspace, nullptr, nullptr,
-                       base + L.dn + (linear_ws(M, H, F, false, sms).part - W8A8_WS_RESERVED), st, &ss)) {
+                       base + L.dn + (linear_ws(M, H, F, false, sms).part - W8A8_WS_RESERVED), st, true, &ss)) {
       W8A8_TRY(ss);
     } else {
       const LinearWs B = linear_ws(M, H, F, false, sms);
@@ -601,6 +611,7 @@ w8a8_status run_ffn(const w8a8_ffn_weights* f, int precision, const uint16_t* X,
       a.y = Y;
       a.partials = base + L.dn + (B.part - W8A8_WS_RESERVED);
       attach_reserved(a, workspace);
+      a.settled = 1;
       W8A8_TRY(launch_stream_gemm(false, a, st));
     }
   }
@@ -641,7 +652,7 @@ extern "C" w8a8_status w8a8_ffn_block(const w8a8_ffn_weights* f, int precision, 
   W8A8_TRY(dev_info(&d));
   const FfnWs L = ffn_ws(M, H, F, d.sms);
   W8A8_TRY(check_ws("w8a8_ffn_block", workspace, ws_bytes, L.total));
-  return run_ffn(f, precision, X, M, Y, h_dbg, workspace, d.sms, as_stream(stream));
+  return run_ffn(f, precision, X, M, Y, h_dbg, workspace, d.sms, as_stream(stream), false);
 }
 
 // --------------------------------------------------------------------------- lm_head
@@ -673,11 +684,11 @@ extern "C" w8a8_status w8a8_lm_head(const w8a8_head_weights* hd, int precision, 
     W8A8_TRY(check_qweight("w8a8_lm_head", &hd->q));
     W8A8_CHECK_ARG(hd->q.n == V && hd->q.k == D, W8A8_ERR_SHAPE, "w8a8_lm_head: weight shape mismatch");
     W8A8_TRY(check_ws("w8a8_lm_head", workspace, ws_bytes, linear_ws(M, V, D, true, d.sms).total));
-    return run_w8a8_linear(&hd->q, X, M, nullptr, EPI_F32, nullptr, logits, top1, nullptr, workspace, d.sms, st);
+    return run_w8a8_linear(&hd->q, X, M, nullptr, EPI_F32, nullptr, logits, top1, nullptr, workspace, d.sms, st, false);
   }
   W8A8_CHECK_ARG(hd->bf16 && aligned16(hd->bf16), W8A8_ERR_INVALID_ARG, "w8a8_lm_head: null or unaligned bf16 table");
   // the tensor-core GEMM's logits need no partial sums
   W8A8_TRY(check_ws("w8a8_lm_head", workspace, ws_bytes,
                     head_bf16_on_tc(M, V, D) ? (size_t)W8A8_WS_RESERVED : linear_ws(M, V, D, false, d.sms).total));
-  return run_bf16_linear(hd->bf16, V, D, X, M, nullptr, EPI_F32, nullptr, logits, top1, workspace, d.sms, st);
+  return run_bf16_linear(hd->bf16, V, D, X, M, nullptr, EPI_F32, nullptr, logits, top1, workspace, d.sms, st, false);
 }

@@ -37,13 +37,20 @@ const char* get_error();
 
 #define W8A8_LAUNCH_CHECK() W8A8_CUDA(cudaGetLastError())
 
-// Programmatic dependent launch.  Kernels of the decoder path are launched with programmatic
-// stream serialization: the next kernel in the stream may start while this one runs, so that it
-// can set up and stream its weights (immutable) early.  Every such kernel calls pdl_wait() before
-// its first read of data an earlier kernel wrote and before its first global write; pdl_wait()
-// returns once the preceding grid has completed and its writes are visible (at once when the
-// launch allowed no overlap).  Because every kernel waits before it can finish, completion is
-// ordered along the whole stream.
+// Programmatic dependent launch.  Kernels are launched with programmatic stream serialization: the
+// next kernel in the stream may start while this one runs, so that it can set up and stream its
+// weights early.  Every such kernel calls pdl_wait() before its first read of data an earlier kernel
+// wrote and before its first global write; pdl_wait() returns once the preceding grid has completed
+// and its writes are visible (at once when the launch allowed no overlap).  Because every kernel
+// waits before it can finish, completion is ordered along the whole stream.
+//
+// What a kernel may read ahead of its wait.  The arguments of a call, weights and scales included, may
+// be the result of any work before it on the stream, and kernels let their dependents start at once, so
+// a call's first launch reads nothing ahead: it waits, and only then triggers its own dependents (its
+// `settled` argument is false).  The call's later launches (settled) cannot start before every CTA of
+// the first one has passed its wait, when all work before the call is complete: they trigger at once and
+// read whatever the call itself does not write ahead of their wait.  The decoder's calls begin with a
+// launch that allows no overlap (set_int), so all of their others are settled.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 // Let the next kernel in the stream begin launching (its CTAs start as resources free up).
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }

@@ -34,7 +34,7 @@ w8a8_status check_fp8_weight(const char* who, const w8a8_fp8_weight* w) {
 // linear's scratch regions start (LinearWs offsets minus the reserved bytes).
 w8a8_status run_fp8_linear(const w8a8_fp8_weight* w, const uint16_t* X, int M, const float* bias, int kind,
                            uint16_t* Y, uint8_t* xq_dbg, float* s_x_dbg, void* ws, char* scratch, int sms,
-                           cudaStream_t st) {
+                           cudaStream_t st, bool settled) {
   const int N = w->n, K = w->k;
   SmallArgs s{};
   s.p = make_small_plan(SMALL_FP8, M, N, K, kind, sms, false);
@@ -43,11 +43,13 @@ w8a8_status run_fp8_linear(const w8a8_fp8_weight* w, const uint16_t* X, int M, c
   float* s_x = reinterpret_cast<float*>(scratch + (L.sx - W8A8_WS_RESERVED));
   if (s.p.ok) {
     if (separate_k1(s.p, K)) {
-      W8A8_TRY(launch_quantize_rows_fp8(X, M, K, w->inv_delta, xq_dbg, s_x, st, reinterpret_cast<uint16_t*>(codes)));
+      W8A8_TRY(launch_quantize_rows_fp8(X, M, K, w->inv_delta, xq_dbg, s_x, st, settled,
+                                        reinterpret_cast<uint16_t*>(codes)));
       if (s_x_dbg) W8A8_CUDA(cudaMemcpyAsync(s_x_dbg, s_x, sizeof(float) * M, cudaMemcpyDeviceToDevice, st));
       s.codes = reinterpret_cast<uint16_t*>(codes);
       s.s_x = s_x;
     }
+    s.settled = settled || s.codes != nullptr;
     s.W = w->wq;
     s.X = X;
     s.M = M;
@@ -65,7 +67,7 @@ w8a8_status run_fp8_linear(const w8a8_fp8_weight* w, const uint16_t* X, int M, c
   }
   W8A8_CHECK_ARG(tc_gemm_supported(M, N, K, kind, false, 0), W8A8_ERR_SHAPE,
                  "fp8 linear: no kernel takes M=%d N=%d K=%d", M, N, K);
-  W8A8_TRY(launch_quantize_rows_fp8(X, M, K, w->inv_delta, reinterpret_cast<uint8_t*>(codes), s_x, st));
+  W8A8_TRY(launch_quantize_rows_fp8(X, M, K, w->inv_delta, reinterpret_cast<uint8_t*>(codes), s_x, st, settled));
   if (xq_dbg) W8A8_CUDA(cudaMemcpyAsync(xq_dbg, codes, (size_t)M * K, cudaMemcpyDeviceToDevice, st));
   if (s_x_dbg) W8A8_CUDA(cudaMemcpyAsync(s_x_dbg, s_x, sizeof(float) * M, cudaMemcpyDeviceToDevice, st));
   TcArgs a{};
@@ -86,6 +88,7 @@ w8a8_status run_fp8_linear(const w8a8_fp8_weight* w, const uint16_t* X, int M, c
   a.err = r.err;
   a.partials = scratch + (L.part - W8A8_WS_RESERVED);
   a.tile_counters = r.tile_counters;
+  a.settled = 1;  // after the quantiser
   return launch_tc_gemm(TC_FP8, a, st);
 }
 
@@ -116,7 +119,7 @@ extern "C" w8a8_status w8a8_fp8_linear(const w8a8_fp8_weight* w, const uint16_t*
   W8A8_TRY(dev_info(&d));
   W8A8_TRY(check_ws_fp8("w8a8_fp8_linear", workspace, ws_bytes, linear_ws(M, w->n, w->k, true, d.sms).total));
   return run_fp8_linear(w, X, M, bias, EPI_BF16, Y, xq_dbg, s_x_dbg, workspace,
-                        reinterpret_cast<char*>(workspace) + W8A8_WS_RESERVED, d.sms, as_stream(stream));
+                        reinterpret_cast<char*>(workspace) + W8A8_WS_RESERVED, d.sms, as_stream(stream), false);
 }
 
 extern "C" w8a8_status w8a8_fp8_ffn_block(const w8a8_fp8_ffn_weights* f, const uint16_t* X, int M, uint16_t* Y,
@@ -143,6 +146,6 @@ extern "C" w8a8_status w8a8_fp8_ffn_block(const w8a8_fp8_ffn_weights* f, const u
   cudaStream_t st = as_stream(stream);
   // gate/up with the GeGLU epilogue into h, then down; disjoint scratch, shared reserved counters
   W8A8_TRY(run_fp8_linear(&f->gate_up, X, M, nullptr, EPI_GEGLU, h, nullptr, nullptr, workspace, base + L.gu, d.sms,
-                          st));
-  return run_fp8_linear(&f->down, h, M, nullptr, EPI_BF16, Y, nullptr, nullptr, workspace, base + L.dn, d.sms, st);
+                          st, false));
+  return run_fp8_linear(&f->down, h, M, nullptr, EPI_BF16, Y, nullptr, nullptr, workspace, base + L.dn, d.sms, st, true);
 }

@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * S, accf0 = full0 + 16 * S, acce0 = accf0 + 8 * NSLOT,
                  done = acce0 + 8 * NSLOT, ready = done + 8;
 
-  pdl_trigger();
+  if (a.settled) pdl_trigger();
   if (warp == kProdWarp && lane == 0) {
     prefetch_tmap(&tmA);
     prefetch_tmap(&tmB);
@@ -474,6 +474,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
+  if (!a.settled) {
+    pdl_wait();
+    pdl_trigger();
+  }
   if (warp != kProdWarp) pdl_wait();  // activations and outputs belong to the preceding kernels
 
   // Persistent: CTA b takes units b, b + grid, ... in the order of TileOrder.
@@ -483,8 +487,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // in uniform registers, which is where the copy and MMA instructions take them from.  Issued by
     // one divergent lane, each instruction's operands were moved there first, and the MMAs waited for
     // their issue: 2048 x 6912 -> 1152 bf16 39.6 -> 31.4 us, W8A8 44.7 -> 31.4.
-    // The weights do not depend on the preceding kernel: those of the first unit's first stages are
-    // requested before the wait for it: 128-token prefill 1704 -> 1650 us (bf16), FP8 FFN block at
+    // The weights do not depend on an earlier launch of this call: those of the first unit's first stages
+    // are requested before the wait for it: 128-token prefill 1704 -> 1650 us (bf16), FP8 FFN block at
     // 512 tokens 36.3 -> 35.6, W8A8 at 64 tokens 33.4 -> 32.9.
     bool ok = true;
     int g = 0, s = 0;  // stages issued; the next one's slot and phase
@@ -874,7 +878,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * S, accf0 = full0 + 16 * S, acce0 = accf0 + 8 * NSLOT,
                  done = acce0 + 8 * NSLOT, ready = done + 8;
 
-  pdl_trigger();
+  if (a.settled) pdl_trigger();
   if (warp == kProdWarp && lane == 0) {
     prefetch_tmap(&tmA);
     prefetch_tmap(&tmB);
@@ -906,6 +910,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
   const uint32_t full_lead = map_to_rank(full0, 0), acce_lead = map_to_rank(acce0, 0);
+  if (!a.settled) {
+    pdl_wait();
+    pdl_trigger();
+  }
   if (warp != kProdWarp) pdl_wait();
 
   if (warp == kProdWarp) {

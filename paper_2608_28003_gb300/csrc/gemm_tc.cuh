@@ -28,6 +28,7 @@ struct TcArgs {
   unsigned int* grid_counter;     // top-1: one counter, zero between calls
   unsigned long long* top_keys;   // top-1: [M] keys, zero between calls
   unsigned int* err;              // device error word
+  int settled;                    // weights may be read ahead of the wait (common.cuh)
   // split-K (few output tiles): the k range of a tile is cut into ksplit parts on different CTAs
   int ksplit;                     // set by the launcher (1: no split)
   int rows_first;                 // set by the launcher: row blocks move fastest over the tiles

@@ -145,7 +145,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
     }
   }
 
-  pdl_trigger();
+  if (a.settled) pdl_trigger();
   if (threadIdx.x == CW * 32) {  // the producer thread: fetch the tensor map before the first copy needs it
     prefetch_tmap(&tmW);
   }
@@ -159,11 +159,15 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
     fence_mbar_init();
   }
   __syncthreads();
+  if (!a.settled) {
+    pdl_wait();
+    pdl_trigger();
+  }
 
   // ------------------------------------------------------------------------ producer thread
   if (warp == CW) {
     if (lane != 0) return;
-    if constexpr (MT > 1) {  // the prologue's constants, which depend on no preceding kernel
+    if constexpr (MT > 1) {  // the prologue's constants, which depend on no launch of this call
       const float* src[3] = {pre ? nullptr : a.inv_delta, a.rn.w_post, a.rn.w_next};
       int n = 0;
 #pragma unroll

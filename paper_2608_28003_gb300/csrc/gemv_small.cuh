@@ -66,6 +66,7 @@ struct SmallArgs {
   int has_rn;              // 1: X is computed from rn (X unused)
   ResNorm rn;
   unsigned int* err;       // device error word
+  int settled;             // weights and constants may be read ahead of the wait (common.cuh)
   SmallPlan p;
   // The FFN's down projection at 5-16 tokens (token slots 8 or 16): the gate/up launch (GeGLU) writes,
   // per CTA and token slot, the maximum of |fl(h * next_inv_delta)| over its h channels (rowmax_out

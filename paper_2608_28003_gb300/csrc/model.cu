@@ -127,9 +127,9 @@ w8a8_status linear(w8a8_model* m, bool int8, const QW& qw, const uint16_t* Wbf, 
                    uint16_t* Y, cudaStream_t st, const ResNorm* rn, const PreCodes* pre = nullptr) {
   if (int8) {
     const w8a8_qweight w = qdesc(qw, N, K);
-    return run_w8a8_linear(&w, X, M, nullptr, 0, Y, nullptr, nullptr, nullptr, m->ws, m->sms, st, rn, pre);
+    return run_w8a8_linear(&w, X, M, nullptr, 0, Y, nullptr, nullptr, nullptr, m->ws, m->sms, st, true, rn, pre);
   }
-  return run_bf16_linear(Wbf, N, K, X, M, nullptr, 0, Y, nullptr, nullptr, m->ws, m->sms, st, rn);
+  return run_bf16_linear(Wbf, N, K, X, M, nullptr, 0, Y, nullptr, nullptr, m->ws, m->sms, st, true, rn);
 }
 
 // At decode the residual step (residual add + the two RMSNorms) runs inside the next linear's
@@ -148,7 +148,8 @@ bool fuse_residual(const w8a8_model* m, int M, bool calib) {
 }
 
 // The decoder over M = B * T rows whose positions start at *m->d_pos (set by the caller; T > 1: the
-// same as start_pos, which a decode step, T = 1, does not read).
+// same as start_pos, which a decode step, T = 1, does not read).  The caller's launch before this one
+// (set_int, or the start of a graph) allows no overlap, so every launch here is settled (common.cuh).
 w8a8_status forward_core(w8a8_model* m, const int32_t* tokens, int B, int T, int start_pos, float* logits, int32_t* top1,
                          bool calib, cudaStream_t st) {
   const w8a8_model_cfg& c = m->cfg;
@@ -223,7 +224,7 @@ w8a8_status forward_core(w8a8_model* m, const int32_t* tokens, int B, int T, int
     const int prec = ffn8 ? W8A8_PREC_W8A8 : W8A8_PREC_BF16;
     if (fuse) {  // the post-attention step inside gate/up
       const ResNorm R{m->y, rc, rn, W.ln_post_attn, W.ln_pre_ffn, c.eps};
-      W8A8_TRY(run_ffn(&f, prec, nullptr, M, m->y, nullptr, m->ws, m->sms, st, &R));
+      W8A8_TRY(run_ffn(&f, prec, nullptr, M, m->y, nullptr, m->ws, m->sms, st, true, &R));
       std::swap(rc, rn);
     } else {
       const bool pre_gu = preq && ffn8;
@@ -233,7 +234,7 @@ w8a8_status forward_core(w8a8_model* m, const int32_t* tokens, int B, int T, int
       if (tr) W8A8_TRY(trace_copy(tr->a_ffn, l, m->a, H, 2));
       uint16_t* h_out = calib ? m->h : nullptr;
       if (tr && tr->h) h_out = tr->h + (size_t)l * tr->max_rows * F;  // the block writes h there
-      W8A8_TRY(run_ffn(&f, prec, m->a, M, m->y, h_out, m->ws, m->sms, st, nullptr, pre_gu ? &pc : nullptr));
+      W8A8_TRY(run_ffn(&f, prec, m->a, M, m->y, h_out, m->ws, m->sms, st, true, nullptr, pre_gu ? &pc : nullptr));
       if (tr) W8A8_TRY(trace_copy(tr->y_f, l, m->y, H, 2));
     }
     if (calib) W8A8_TRY(launch_act_absmax(m->h, M, F, m->stat_down(l), st));
@@ -257,9 +258,9 @@ w8a8_status forward_core(w8a8_model* m, const int32_t* tokens, int B, int T, int
     int32_t* tp = top1 + r0;
     if (lm8) {
       const w8a8_qweight w = qdesc(m->q_lm, c.vocab, H);
-      W8A8_TRY(run_w8a8_linear(&w, X, rows, nullptr, 2, nullptr, lg, tp, nullptr, m->ws, m->sms, st));
+      W8A8_TRY(run_w8a8_linear(&w, X, rows, nullptr, 2, nullptr, lg, tp, nullptr, m->ws, m->sms, st, true));
     } else {
-      W8A8_TRY(run_bf16_linear(m->embed, c.vocab, H, X, rows, nullptr, 2, nullptr, lg, tp, m->ws, m->sms, st));
+      W8A8_TRY(run_bf16_linear(m->embed, c.vocab, H, X, rows, nullptr, 2, nullptr, lg, tp, m->ws, m->sms, st, true));
     }
   }
   return W8A8_OK;

@@ -18,9 +18,8 @@ namespace w8a8 {
 // ------------------------------------------------------------------------------ K1
 // One CTA per row.  Each thread holds up to kVec 16-byte vectors (8 bf16 each) of the row in
 // registers between the max pass and the quantise pass; longer rows are re-read.
-// 1 / delta, part of the prepared weight (as in the decode GEMV, which reads it there too; no kernel that
-// writes it lets its dependents start early), is read ahead of the wait for the kernel that produces X, and the
-// row's loads are issued together: W8A8 FFN block at 17 tokens 29.6 -> 27.4 us, at 64 32.9 -> 30.7 (all loads
+// In a launch that is not its call's first (settled) 1 / delta, part of the prepared weight, is read ahead of the
+// wait for the kernel that produces X; the row's loads are issued together: W8A8 FFN block at 17 tokens 29.6 -> 27.4 us, at 64 32.9 -> 30.7 (all loads
 // behind the wait: 31.9), at 512 57.2 -> 54.8, at 4096 171.4 -> 168.7; FP8 at 512 37.1 -> 35.2.  Latency bounds it
 // up to a few hundred rows; 6912 x 2048 (56 MB in and out, 8.3 us at the copy rate) takes 16 us.
 template <int kVec, bool kFp8>
@@ -28,7 +27,9 @@ __global__ void __launch_bounds__(256) quantize_rows_kernel(const uint16_t* __re
                                                            const float* __restrict__ inv_delta,
                                                            int8_t* __restrict__ xq,
                                                            uint16_t* __restrict__ xq_f16,
-                                                           float* __restrict__ s_x, int* __restrict__ qsum) {
+                                                           float* __restrict__ s_x, int* __restrict__ qsum,
+                                                           int settled) {
+  if (!settled) pdl_wait();
   pdl_trigger();
   const int row = blockIdx.x;
   const int nvec = K >> 3;
@@ -167,12 +168,12 @@ __global__ void __launch_bounds__(256) quantize_rows_kernel(const uint16_t* __re
 }
 
 w8a8_status launch_quantize_rows(const uint16_t* X, int M, int K, const float* inv_delta, int8_t* xq,
-                                 uint16_t* xq_f16, float* s_x, cudaStream_t st, int* qsum) {
+                                 uint16_t* xq_f16, float* s_x, cudaStream_t st, bool settled, int* qsum) {
   if (M == 0) return W8A8_OK;
   const int nvec = K / 8;
   const int threads = nvec <= 4 * 128 ? 128 : 256;
   W8A8_CUDA(launch_pdl(quantize_rows_kernel<4, false>, dim3(M), dim3(threads), 0, st, X, K, inv_delta, xq, xq_f16,
-                       s_x, qsum));
+                       s_x, qsum, (int)settled));
   return W8A8_OK;
 }
 
@@ -226,12 +227,12 @@ w8a8_status launch_quantize_known_rows(const uint16_t* X, int M, int K, const fl
 }
 
 w8a8_status launch_quantize_rows_fp8(const uint16_t* X, int M, int K, const float* inv_delta, uint8_t* xq,
-                                     float* s_x, cudaStream_t st, uint16_t* xq_f16) {
+                                     float* s_x, cudaStream_t st, bool settled, uint16_t* xq_f16) {
   if (M == 0) return W8A8_OK;
   const int nvec = K / 8;
   const int threads = nvec <= 4 * 128 ? 128 : 256;
   W8A8_CUDA(launch_pdl(quantize_rows_kernel<4, true>, dim3(M), dim3(threads), 0, st, X, K, inv_delta,
-                       reinterpret_cast<int8_t*>(xq), xq_f16, s_x, static_cast<int*>(nullptr)));
+                       reinterpret_cast<int8_t*>(xq), xq_f16, s_x, static_cast<int*>(nullptr), (int)settled));
   return W8A8_OK;
 }
 
@@ -533,7 +534,7 @@ extern "C" w8a8_status w8a8_quantize_activations(const uint16_t* X, int M, int K
                  W8A8_ERR_ALIGN, "w8a8_quantize_activations: pointers must be 16-byte aligned");
   w8a8_status s = check_device();
   if (s != W8A8_OK) return s;
-  return launch_quantize_rows(X, M, K, inv_delta, xq, xq_f16, s_x, as_stream(stream), nullptr);
+  return launch_quantize_rows(X, M, K, inv_delta, xq, xq_f16, s_x, as_stream(stream), false, nullptr);
 }
 
 // ------------------------------------------------------------------------ FP8 (e4m3) variant
@@ -582,5 +583,5 @@ extern "C" w8a8_status w8a8_fp8_quantize_activations(const uint16_t* X, int M, i
                  "w8a8_fp8_quantize_activations: pointers must be 16-byte aligned");
   w8a8_status s = check_device();
   if (s != W8A8_OK) return s;
-  return launch_quantize_rows_fp8(X, M, K, inv_delta, xq, s_x, as_stream(stream), nullptr);
+  return launch_quantize_rows_fp8(X, M, K, inv_delta, xq, s_x, as_stream(stream), false, nullptr);
 }

@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(kThreads, Cps<NB>::value)
   const long long u1 = p.whole ? (long long)(cta + 1) * ZG / P * C : (long long)(cta + 1) * U / P;
   auto cta_of = [&](long long u) -> int { return (int)(((u + 1) * P + U - 1) / U - 1); };
 
-  pdl_trigger();
+  if (a.settled) pdl_trigger();
   if (threadIdx.x == kConsumerWarps * 32) {  // the producer thread: fetch the tensor maps before the first copy needs them
     prefetch_tmap(&tmW);
     prefetch_tmap(&tmX);
@@ -140,6 +140,10 @@ __global__ void __launch_bounds__(kThreads, Cps<NB>::value)
     fence_mbar_init();
   }
   __syncthreads();
+  if (!a.settled) {
+    pdl_wait();
+    pdl_trigger();
+  }
   if (u0 >= u1) {
     pdl_wait();
     return;
@@ -164,7 +168,7 @@ __global__ void __launch_bounds__(kThreads, Cps<NB>::value)
       for (int b = 0; b < BSTEPS; ++b)
         tma_load_2d(ring + (uint32_t)slot * SB + kBox + b * XBOX, &tmX, ch * KC + h * BOXK + b * 64, z * TOK, bar);
     };
-    // The weights of the first slots do not depend on the preceding kernel: request them before
+    // The weights of the first slots do not depend on an earlier launch of this call: request them before
     // waiting for it, then add the token rows of X to the same slots.
     int npre = 0;
     for (long long u = u0; u < u1 && npre < S; ++u)
@@ -618,7 +622,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   const long long u1 = p.whole ? (long long)(cta + 1) * G / P * C : (long long)(cta + 1) * U / P;
   auto cta_of = [&](long long u) -> int { return (int)(((u + 1) * P + U - 1) / U - 1); };
 
-  pdl_trigger();
+  if (a.settled) pdl_trigger();
   if (threadIdx.x == kConsumerWarps * 32) {  // the producer thread: fetch the tensor map before the first copy needs it
     prefetch_tmap(&tmW);
   }
@@ -630,12 +634,16 @@ __global__ void __launch_bounds__(kThreads, 2)
     fence_mbar_init();
   }
   __syncthreads();
+  if (!a.settled) {
+    pdl_wait();
+    pdl_trigger();
+  }
   if (u0 >= u1) {
     pdl_wait();
     return;
   }
 
-  // The producer streams weights only (independent of the preceding kernel) and starts at once;
+  // The producer streams weights only (which depend on no launch of this call) and starts at once;
   // the consumers wait for the preceding kernel, then stage the activation codes.
   if (warp == kConsumerWarps) {  // ---------------------------------------------- producer thread
     if (lane != 0) return;

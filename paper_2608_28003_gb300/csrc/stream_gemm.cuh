@@ -47,6 +47,7 @@ struct StreamArgs {
   unsigned int* grid_counter;      // one counter (top-1)
   unsigned long long* top_keys;    // [M]
   unsigned int* err;               // device error word
+  int settled;                     // weights may be read ahead of the wait (common.cuh)
 };
 
 StreamPlan make_stream_plan(bool int8_weights, int M, int N, int K, int sm_count);
