@@ -180,15 +180,18 @@ bool decode_gemv_takes(bool int8, int M, int N, int K, bool geglu, int sms) {
 // rules hold (W8A8: the weights' fp16 code copy must exist); false leaves them to the streaming
 // kernel.  Below 64 tokens a 128-token tile is mostly padding; it still beats the streaming kernel
 // on the decoder's linears (one wave of 128 x 64 tiles, measured 12-15 us against 20 us at M 16) and,
-// on lm_head-sized outputs (262144 x 1152), wherever both read the same bytes or the streaming kernel's
-// arithmetic is the bound: bf16 at 1 token 92.5 us against 94.7, at 16 96.7 / 102, at 32 100 / 118, at
-// 63 104 / 277; W8A8 at 17 tokens 104 / 117, at 33 107 / 276.  W8A8 at up to 16 tokens stays with the
-// streaming kernel, which reads the INT8 codes, half the bytes of their fp16 copy (16 tokens 81 / 103).
-constexpr int kTcMinTokensWideInt8 = 17, kTcMinTokensWideBf16 = 1, kTcMinTokensNarrow = 9, kTcNarrowMaxN = 16384;
+// on lm_head-sized outputs (262144 x 1152) from 17 tokens, where the streaming kernel's arithmetic is the
+// bound: bf16 at 17 tokens 99 us / 117, at 33 103 / 254, at 63 106 / 279; W8A8 at 17 104 / 117, at 33 107 /
+// 276.  Up to 16 tokens both stay with the streaming kernel: W8A8 because it reads the INT8 codes, half the
+// bytes of their fp16 copy (16 tokens 81 / 103), bf16 because it sums k in up to four chains per output, which
+// one tensor-memory accumulator does not: relative error of the logits against 64 bits 2.5e-7 at 1-8 tokens
+// and 5.4e-7 at 9-16, where the GEMM has 1.1e-6 and saves 2-5 % (8 tokens 101 us / 98, 16 106 / 99); from 17
+// tokens the streaming kernel has one chain and 1.1e-6 too.
+constexpr int kTcMinTokensWide = 17, kTcMinTokensNarrow = 9, kTcNarrowMaxN = 16384;
 
 // Whether a bf16 lm_head call runs the tensor-core GEMM (tc_path's rule for logits).
 static bool head_bf16_on_tc(int M, int N, int K) {
-  return M >= (N <= kTcNarrowMaxN ? kTcMinTokensNarrow : kTcMinTokensWideBf16) &&
+  return M >= (N <= kTcNarrowMaxN ? kTcMinTokensNarrow : kTcMinTokensWide) &&
          tc_gemm_supported(M, N, K, EPI_F32, true, max_top_keys());
 }
 
@@ -196,7 +199,7 @@ static bool tc_path(bool int8, const void* W16, const uint16_t* X, int M, int N,
                     const float* inv_delta, const float* s_w, uint16_t* Y, float* logits, int32_t* top1,
                     const w8a8_debug* dbg, void* ws, void* codes, float* s_x, void* part, cudaStream_t st,
                     bool settled, w8a8_status* status, const PreCodes* pre = nullptr) {
-  if (M < (N <= kTcNarrowMaxN ? kTcMinTokensNarrow : int8 ? kTcMinTokensWideInt8 : kTcMinTokensWideBf16) || !W16 ||
+  if (M < (N <= kTcNarrowMaxN ? kTcMinTokensNarrow : kTcMinTokensWide) || !W16 ||
       !tc_gemm_supported(M, N, K, kind, top1 != nullptr, max_top_keys()))
     return false;
   TcArgs a{};

@@ -1,5 +1,6 @@
-"""lm_head-sized outputs at few tokens on the tensor-core GEMM: bf16 from one token, W8A8 from 17, on both
-sides of the line and at a ragged vocabulary, logits and top-1 against the oracle."""
+"""lm_head-sized outputs at few tokens: the streaming kernel to 16, the tensor-core GEMM from 17, on both
+sides of the line and at a ragged vocabulary, logits and top-1 against the oracle, and the precision of the
+bf16 logits that the line keeps."""
 import numpy as np
 import pytest
 import torch
@@ -68,3 +69,18 @@ def test_bf16_head_runs_in_the_queried_workspace(M, vocab):
     lg = logits.cpu().numpy()
     assert np.all(np.abs(lg - r["logits"]) <= 1152 * 2.0 ** -24 * mag + 1e-30)
     assert np.array_equal(top1.cpu().numpy(), lg.argmax(axis=1))
+
+
+@pytest.mark.parametrize("M,bound", [(1, 4e-7), (5, 4e-7), (8, 4e-7), (9, 8e-7), (16, 8e-7)])
+def test_bf16_logits_keep_the_split_sums(M, bound):
+    """Relative error against 64 bits: four chains per output to 8 tokens (measured 2.5e-7) and two to 16
+    (5.4e-7); one accumulator over all of K has 1.1e-6."""
+    from paper_2608_28003_gb300 import build
+    build.build()
+    from paper_2608_28003_gb300 import binding as B
+    g = torch.Generator("cuda").manual_seed(M)
+    w = (torch.randn(32768, 1152, device="cuda", generator=g) * 0.02).to(torch.bfloat16)
+    x = torch.randn(M, 1152, device="cuda", generator=g).to(torch.bfloat16)
+    logits, _ = B.lm_head(B.HeadWeights(32768, 1152, bf16=w), B.W8A8_PREC_BF16, x)
+    want = x.double() @ w.double().t()
+    assert float((logits.double() - want).norm() / want.norm()) <= bound
