@@ -195,6 +195,13 @@ static bool head_bf16_on_tc(int M, int N, int K) {
          tc_gemm_supported(M, N, K, EPI_F32, true, max_top_keys());
 }
 
+// Workspace of a bf16 lm_head call: neither the tensor-core GEMM's logits nor a streaming plan that splits no
+// row group (every vocabulary of 128 rows per CTA or more) has partial sums.
+static size_t head_bf16_ws(int M, int N, int K, int sms) {
+  if (head_bf16_on_tc(M, N, K) || make_stream_plan(false, M, N, K, sms).whole) return W8A8_WS_RESERVED;
+  return linear_ws(M, N, K, false, sms).total;
+}
+
 static bool tc_path(bool int8, const void* W16, const uint16_t* X, int M, int N, int K, const float* bias, int kind,
                     const float* inv_delta, const float* s_w, uint16_t* Y, float* logits, int32_t* top1,
                     const w8a8_debug* dbg, void* ws, void* codes, float* s_x, void* part, cudaStream_t st,
@@ -661,9 +668,7 @@ extern "C" w8a8_status w8a8_ffn_block(const w8a8_ffn_weights* f, int precision, 
 // --------------------------------------------------------------------------- lm_head
 extern "C" w8a8_status w8a8_lm_head_workspace_size(int M, int vocab, int hidden, size_t* bytes) {
   W8A8_CHECK_ARG(bytes && M >= 0 && vocab >= 0 && hidden >= 0, W8A8_ERR_INVALID_ARG, "w8a8_lm_head_workspace_size: bad argument");
-  *bytes = linear_ws(M, vocab, hidden, true, device_sms()).total;
-  // a bf16 call that the streaming kernel takes may need more for its partial sums
-  if (!head_bf16_on_tc(M, vocab, hidden)) *bytes = std::max(*bytes, linear_ws(M, vocab, hidden, false, device_sms()).total);
+  *bytes = std::max(linear_ws(M, vocab, hidden, true, device_sms()).total, head_bf16_ws(M, vocab, hidden, device_sms()));
   return W8A8_OK;
 }
 
@@ -690,8 +695,6 @@ extern "C" w8a8_status w8a8_lm_head(const w8a8_head_weights* hd, int precision, 
     return run_w8a8_linear(&hd->q, X, M, nullptr, EPI_F32, nullptr, logits, top1, nullptr, workspace, d.sms, st, false);
   }
   W8A8_CHECK_ARG(hd->bf16 && aligned16(hd->bf16), W8A8_ERR_INVALID_ARG, "w8a8_lm_head: null or unaligned bf16 table");
-  // the tensor-core GEMM's logits need no partial sums
-  W8A8_TRY(check_ws("w8a8_lm_head", workspace, ws_bytes,
-                    head_bf16_on_tc(M, V, D) ? (size_t)W8A8_WS_RESERVED : linear_ws(M, V, D, false, d.sms).total));
+  W8A8_TRY(check_ws("w8a8_lm_head", workspace, ws_bytes, head_bf16_ws(M, V, D, d.sms)));
   return run_bf16_linear(hd->bf16, V, D, X, M, nullptr, EPI_F32, nullptr, logits, top1, workspace, d.sms, st, false);
 }

@@ -53,7 +53,7 @@ def test_split_line_of_short_k_ranges(M, K):
     assert np.array_equal(y.float().cpu().numpy(), r["y"])
 
 
-@pytest.mark.parametrize("vocab", [16400, 16392, 600])  # tensor cores; streaming kernel (V not a multiple of 16; few rows)
+@pytest.mark.parametrize("vocab", [16400, 16392, 600, 40960])  # ragged, not a multiple of 16, few rows; no split row group
 @pytest.mark.parametrize("M", [1, 4, 8])
 def test_bf16_head_runs_in_the_queried_workspace(M, vocab):
     from paper_2608_28003_gb300 import build
