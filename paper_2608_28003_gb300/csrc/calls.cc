@@ -93,6 +93,18 @@ bool shape_of(PyObject* t, int n, long long* out) {
     if (!as_int(PySequence_GetItem(s.p, i), out + i)) return false;
   return true;
 }
+// the extents of a matrix: a tensor of more dimensions is refused, not read as its first two
+bool matrix_shape(PyObject* t, long long* out) {
+  Ref s(PyObject_GetAttr(t, s_shape));
+  if (!s) return false;
+  const Py_ssize_t dims = PySequence_Size(s.p);
+  if (dims < 0) return false;
+  if (dims > 2) {
+    PyErr_Format(PyExc_ValueError, "a matrix expected, not a tensor of %zd dimensions", dims);
+    return false;
+  }
+  return shape_of(t, 2, out);
+}
 // The binding's rule for an input: a contiguous CUDA tensor.
 bool check_bits(PyObject* t) {
   Ref c(PyObject_GetAttr(t, s_is_cuda));
@@ -258,7 +270,7 @@ PyObject* py_linear_bf16(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (!nargs_are(n, 6, "linear_bf16")) return nullptr;
   long long nk[2], M;
   size_t need = 0;
-  if (!shape_of(a[0], 2, nk) || !shape_of(a[1], 1, &M)) return nullptr;
+  if (!matrix_shape(a[0], nk) || !shape_of(a[1], 1, &M)) return nullptr;
   Ref y;
   if (a[3] == Py_None) {
     y.p = new_empty(a[1], M, nk[0], g_bf16);

@@ -48,6 +48,8 @@ def test_wrong_objects_raise(B):
         B.ffn_block(None, 1, x, ws=ws)
     with pytest.raises((IndexError, TypeError)):
         B.linear_bf16(torch.zeros(16), x, ws=ws)
+    with pytest.raises(ValueError):
+        B.linear_bf16(torch.zeros(4, 16, 32, dtype=torch.bfloat16), x, ws=ws)
 
 
 @pytest.mark.gpu
