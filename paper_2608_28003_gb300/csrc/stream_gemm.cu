@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(kThreads, Cps<NB>::value)
           float m = max_nan(live && ina ? ya : -INFINITY, live && inb ? yb : -INFINITY);
 #pragma unroll
           for (int o = 4; o < 32; o <<= 1) m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, o));
-          if (__any_sync(0xffffffffu, !(m < known[nb][h]))) {
+          if (__any_sync(0xffffffffu, live && !(m < known[nb][h]))) {  // slots past M never vote
             unsigned long long best = 0ull;
             auto offer = [&](float y, int i) {
               const unsigned long long key =
