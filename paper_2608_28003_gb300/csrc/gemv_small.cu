@@ -167,7 +167,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
   // ------------------------------------------------------------------------ producer thread
   if (warp == CW) {
     if (lane != 0) return;
-    if constexpr (MT > 1) {  // the prologue's constants, which depend on no launch of this call
+    if constexpr (MT > 4) {  // the prologue's constants, which depend on no launch of this call
       const float* src[3] = {pre ? nullptr : a.inv_delta, a.rn.w_post, a.rn.w_next};
       int n = 0;
 #pragma unroll
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
   // weights of the fused residual norm (constants): this thread's 8 channels
   const int nvk = a.K >> 3;
   float wp[8], wn[8];
-  if (kRn && MT == 1 && a.has_rn && tid < nvk) {
+  if (kRn && MT <= 4 && a.has_rn && tid < nvk) {
     const float4* p0 = reinterpret_cast<const float4*>(a.rn.w_post + 8 * tid);
     const float4* p1 = reinterpret_cast<const float4*>(a.rn.w_next + 8 * tid);
     const float4 a0 = p0[0], a1 = p0[1], b0 = p1[0], b1 = p1[1];
@@ -309,9 +309,10 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
   if (kRn && a.has_rn) {
     uint16_t* as = kQ ? reinterpret_cast<uint16_t*>(xsp + p.xbytes) : reinterpret_cast<uint16_t*>(xsp);
     const int astride = kQ ? kpad : xsb;  // elements between the rows in shared memory
-    if constexpr (MT == 1) {
-      {
-        constexpr int m = 0;
+    if constexpr (MT <= 4) {
+      // Up to four token slots: all threads on one row after the other, two block sums a row, in the order of
+      // the stand-alone kernel.  (A warp per row leaves most warps idle here: decode of 2 sequences 691 -> 771 us.)
+      for (int m = 0; m < MT; ++m) {
         const bool mine = m < a.M && tid < nvk;
         float yv[8], rv[8];
         float ss = 0.0f;
@@ -321,13 +322,13 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
           const float4* rp = reinterpret_cast<const float4*>(a.rn.r_in + (size_t)m * a.K + 8 * tid);
           const float4 r0 = rp[0], r1 = rp[1];
           rv[0] = r0.x; rv[1] = r0.y; rv[2] = r0.z; rv[3] = r0.w; rv[4] = r1.x; rv[5] = r1.y; rv[6] = r1.z; rv[7] = r1.w;
-  #pragma unroll
+#pragma unroll
           for (int e = 0; e < 8; ++e) ss += yv[e] * yv[e];
         }
         const float inv_y = 1.0f / sqrtf(consumer_sum(ss, s_red, warp, lane) / (float)a.K + a.rn.eps);
         float ss2 = 0.0f;
         if (mine) {
-  #pragma unroll
+#pragma unroll
           for (int e = 0; e < 8; ++e) {
             rv[e] += yv[e] * inv_y * wp[e];
             ss2 += rv[e] * rv[e];
@@ -343,18 +344,18 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
           uint4 w = make_uint4(0u, 0u, 0u, 0u);
           if (mine) {
             float o[8];
-  #pragma unroll
+#pragma unroll
             for (int e = 0; e < 8; ++e) o[e] = rv[e] * inv_r * wn[e];
             w.x = (uint32_t)f32_to_bf16_bits(o[0]) | ((uint32_t)f32_to_bf16_bits(o[1]) << 16);
             w.y = (uint32_t)f32_to_bf16_bits(o[2]) | ((uint32_t)f32_to_bf16_bits(o[3]) << 16);
             w.z = (uint32_t)f32_to_bf16_bits(o[4]) | ((uint32_t)f32_to_bf16_bits(o[5]) << 16);
             w.w = (uint32_t)f32_to_bf16_bits(o[6]) | ((uint32_t)f32_to_bf16_bits(o[7]) << 16);
           }
-          *reinterpret_cast<uint4*>(as + (size_t)m * (kQ ? kpad : xsb) + 8 * tid) = w;
+          *reinterpret_cast<uint4*>(as + (size_t)m * astride + 8 * tid) = w;
         }
       }
     } else {
-      // Several token slots: a warp per row, so that the rows run side by side and their sums need no
+      // Eight token slots: a warp per row, so that the rows run side by side and their sums need no
       // block barrier.  (All 256 threads on one row after the other took about 1 us per slot, two
       // launches a layer: decode of 8 sequences 1170 us, now 1070.)  Lane l owns the 16-byte vectors
       // l, l + 32, ...; the first kKeep of them stay in registers (K <= 1280: all), later ones are
@@ -464,10 +465,10 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
         const bool live = m < a.M;
         if (live) {
           const uint4* src = reinterpret_cast<const uint4*>(xrows + (size_t)m * xstride);
-          // 1-2 slots: the row's loads together ahead of their use (W8A8 6912 -> 1152 at 1 token 4.8 -> 4.4
-          // us, a decode step 577 -> 573); at 4 slots that made short rows slower (1152 -> 1536 5.1 -> 5.5)
+          // 1 slot: the row's loads together ahead of their use (W8A8 6912 -> 1152 at 1 token 4.8 -> 4.4 us); at
+          // 2 and 4 slots that made short rows slower (1152 -> 1536 at 2 3.5 -> 4.1, at 4 5.1 -> 5.5)
           uint4 xw[4];
-          if constexpr (MT <= 2) {
+          if constexpr (MT == 1) {
 #pragma unroll
             for (int v = 0; v < 4; ++v)
               if (tid + v * CW * 32 < nvec) xw[v] = src[tid + v * CW * 32];
@@ -476,7 +477,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
           for (int v = 0; v < 4; ++v) {
             const int vi = tid + v * CW * 32;
             if (vi < nvec) {
-              const uint4 w = MT <= 2 ? xw[v] : src[vi];
+              const uint4 w = MT == 1 ? xw[v] : src[vi];
               const float4 d0 = idr[v][0], d1 = idr[v][1];
               xh[v][0] = __fmul_rn(bf16_lo(w.x), d0.x);
               xh[v][1] = __fmul_rn(bf16_hi(w.x), d0.y);
@@ -1127,7 +1128,7 @@ SmallPlan make_small_plan(int wkind, int M, int N, int K, int kind, int sm_count
   p.smem_bytes = 1024 + p.stages * p.stage_bytes + p.xbytes + p.abytes + p.rbytes + 16 * p.stages;
   // the prologue's constants: first into the partial sums' place, then past the end as far as the SM's
   // CTAs leave room
-  const bool want[3] = {mma && int8_weights && p.MT < 16, fused_norm && p.MT > 1, fused_norm && p.MT > 1};
+  const bool want[3] = {mma && int8_weights && p.MT < 16, fused_norm && p.MT > 4, fused_norm && p.MT > 4};
   int used = 0;
   for (int i = 0; i < 3; ++i) {
     p.coff[i] = -1;
