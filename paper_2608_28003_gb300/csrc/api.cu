@@ -126,7 +126,7 @@ static bool small_gemv(bool int8, const void* W, const float* inv_delta, const f
   if (!a.p.ok) return false;
   // The quantiser's own launch writes `codes` and `s_x`, unless the producer of X has written its codes.
   const bool known = rm && rm->in;
-  if (int8 && codes && !rn && separate_k1(a.p, K)) {
+  if (int8 && codes && !rn && separate_k1(a.p, M, K)) {
     if (pre && pre->codes16 && !dbg) {
       a.codes = pre->codes16;
       a.s_x = pre->s_x;

@@ -6,7 +6,7 @@
 // epilogue dequantises y = fl32(fl32(s_x s_w) * acc) (+ bias), the order of Eq. gemm-final.
 //
 // Routing: 1-16 tokens run the row-owning decode GEMV on its tensor-core path where it takes the shape
-// (e4m3 weights and codes widened to fp16; K1 fused, or a launch before it at 9-16 tokens or a long K);
+// (e4m3 weights and codes widened to fp16; K1 fused or a launch before it, see separate_k1);
 // other calls run the per-token quantiser, then the tcgen05 GEMM
 // with kind::f8f6f4 on the one-byte codes (no wider copy of the weights exists or is needed).
 #include "common.cuh"
@@ -42,7 +42,7 @@ w8a8_status run_fp8_linear(const w8a8_fp8_weight* w, const uint16_t* X, int M, c
   char* codes = scratch + (L.xf16 - W8A8_WS_RESERVED);
   float* s_x = reinterpret_cast<float*>(scratch + (L.sx - W8A8_WS_RESERVED));
   if (s.p.ok) {
-    if (separate_k1(s.p, K)) {
+    if (separate_k1(s.p, M, K)) {
       W8A8_TRY(launch_quantize_rows_fp8(X, M, K, w->inv_delta, xq_dbg, s_x, st, settled,
                                         reinterpret_cast<uint16_t*>(codes)));
       if (s_x_dbg) W8A8_CUDA(cudaMemcpyAsync(s_x_dbg, s_x, sizeof(float) * M, cudaMemcpyDeviceToDevice, st));

@@ -87,11 +87,18 @@ SmallPlan make_small_plan(int wkind, int M, int N, int K, int kind, int sm_count
 
 // Whether the codes of a W8A8 or FP8 call (without a fused residual norm) come from a launch before the
 // GEMV.  Every CTA of the GEMV needs all of them, so where its own pass over the rows takes longer than a
-// launch of the quantiser, that is faster: W8A8 1152 -> 6912 at 16 tokens 11.0 -> 9.5 us, 6912 -> 1152 at 8
-// tokens 11.4 -> 9.0, the FFN block at 8 tokens 20.2 -> 18.9.  At 5-8 tokens and K = 1152 the pass takes
-// under 2 us, less than a launch (1152 -> 6912: 7.6 us with it).  The line lies between those two lengths.
-constexpr int kSeparateK1MinK = 4096;
-inline bool separate_k1(const SmallPlan& p, int K) { return p.MT == 16 || (p.MT == 8 && K >= kSeparateK1MinK); }
+// launch of the quantiser, that is faster: always at 9-16 tokens (W8A8 at 9 tokens 1024 -> 1152 8.8 -> 5.0 us,
+// 1152 -> 6912 12.9 -> 8.2), and at 8 slots by the elements a warp has to pass over, M K with a warp per row and half
+// of that with two (16 consumer warps).  Both sides measured at 3, 5 and 8 tokens, K of 256 to 3584 and
+// 1024, 2304 and 6912 outputs (us in the GEMV / with the launch):
+//   8 warps:  768 -> 2304 at 8 tokens W8A8 4.9 / 4.8, FP8 5.6 / 4.6; 1152 -> 6912 at 8 7.3 / 6.8, 7.0 / 6.5, at 5 6.6 / 6.9,
+//             6.3 / 6.5; 1280 -> 2304 at 5 5.4 / 5.4, 6.3 / 5.2; 2048 -> 2304 at 8 7.5 / 5.7, 9.5 / 5.6;
+//   16 warps: 1536 -> 1024 at 8 4.6 / 4.6, 4.4 / 4.4; 2048 -> 1024 at 8 5.2 / 4.9, 5.1 / 4.6, at 5 4.6 / 4.9, 4.5 / 4.6; 3584 ->
+//             1024 at 8 7.0 / 6.1, 6.9 / 5.5, at 5 6.1 / 6.3, 6.0 / 5.8.
+constexpr int kSeparateK1Elems = 6144, kSeparateK1Elems16Warps = 16384;
+inline bool separate_k1(const SmallPlan& p, int M, int K) {
+  return p.MT == 16 || (p.MT == 8 && (long long)M * K >= (p.cw == 16 ? kSeparateK1Elems16Warps : kSeparateK1Elems));
+}
 w8a8_status launch_small_gemv(int wkind, const SmallArgs& a, cudaStream_t st);
 
 }  // namespace w8a8
