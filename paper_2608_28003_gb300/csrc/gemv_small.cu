@@ -1142,6 +1142,12 @@ SmallPlan make_small_plan(int wkind, int M, int N, int K, int kind, int sm_count
       p.cextra += bytes;
     }
   }
+  // bf16 at 1-4 slots takes so few registers that three CTAs fit on an SM.  With 1.5 to 2 CTAs per SM in the grid, the
+  // next call's then crowd on some SMs and leave others one short: kept to two (2048 -> 2048 at 3 tokens
+  // 5.05 -> 4.04 us, 1152 -> 2304 at 2 3.41 -> 2.97; no difference below 1.2 CTAs per SM, and at 192 CTAs three
+  // are better, 1152 -> 1536 at 3 3.32 against 3.51).
+  if (wkind == SMALL_BF16 && p.MT <= 4 && !fused_norm && 2 * p.P > 3 * sm_count)
+    p.cextra = std::max(0, kSmemLimit / 3 + 1024 - p.smem_bytes);
   p.ok = 1;
   return p;
 }

@@ -35,7 +35,7 @@ struct SmallPlan {
   // the activations (in the partial sums' place, free until the end, or past smem_bytes), -1: read
   // from global memory
   int coff[3];
-  int cextra;       // dynamic shared memory past smem_bytes
+  int cextra;       // dynamic shared memory past smem_bytes: constants, or none of them and only a bound on the CTAs per SM
 };
 
 // The decoder's residual step in front of a decode linear, fused into the GEMV's prologue:
