@@ -597,9 +597,10 @@ w8a8_status launch_attention_prefill(const PrefillOperands& w, const AttnShape& 
   W8A8_TRY(make_tmap_2d(&tq, w.q, 2, qw, (uint64_t)s.B * s.T, qw * 2, 64, kBq, 128));
   W8A8_TRY(make_tmap_2d(&tk, w.k, 2, kHd, kv * keys_pad, kHd * 2, 64, kBk, 128));
   W8A8_TRY(make_tmap_2d(&tv, w.vt, 2, (uint64_t)keys_pad, kv * kHd, (uint64_t)keys_pad * 2, 64, kHd, 128));
-  // two CTAs per query block while that leaves none of them waiting for an SM (2048 tokens: 64 blocks)
+  // two CTAs per query block while that leaves none of them waiting for an SM (2048 tokens: 64 blocks) and there is
+  // more than one key tile to share
   const long long blocks = (long long)((s.T + kBq - 1) / kBq) * s.n_q * s.B;
-  return 2 * blocks <= sms ? launch_split<2>(tq, tk, tv, s, pos0, keys_pad, o, err, st)
+  return 2 * blocks <= sms && pos0 + s.T > kBk ? launch_split<2>(tq, tk, tv, s, pos0, keys_pad, o, err, st)
                            : launch_split<1>(tq, tk, tv, s, pos0, keys_pad, o, err, st);
 }
 
