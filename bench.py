@@ -3,7 +3,7 @@
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--quick]
 
-Prints ONE JSON line (rank 0).  The headline workload is decode of a 26-layer Gemma-3-1B-shaped
+Prints ONE JSON line (rank 0) to stdout, and its tables as another to stderr.  The headline workload is decode of a 26-layer Gemma-3-1B-shaped
 decoder (random-init bf16 weights, hidden 1152, 4 query / 1 KV heads of 256, FFN 6912, vocab
 262144) under the precision mask "FFN 5+5 + lm_head" (the FFN blocks of the five outermost
 layers at each end and lm_head in W8A8, everything else bf16), batch 1: a 128-token prefill,
@@ -12,7 +12,7 @@ included).  Tokens are seeded uniform ids, teacher-forced.  Every step streams a
 weights, far more than the 129 MB L2, so no flush is needed between steps.  ``value`` = ms per
 decoded token of the whole job (time, max over ranks, / tokens all ranks decoded; replicas only).
 
-The same line carries:
+The tables on stderr:
   * ``masks``: per-mask decode ms/token, the latency change against the all-bf16 mask, Top-1
     agreement and perplexity change, for the 16 candidate masks, and the mask the library's
     allocator picks (Top-1 >= 98.9 %, perplexity change <= 1 %);
@@ -21,6 +21,8 @@ The same line carries:
   * ``kernels``: per-call time, TOPS and algorithmic GB/s of the single W8A8 linear (M = 16,
     1152 -> 6912), the FFN block (M in 1, 8, 64, 512, 2048) and lm_head (M in 1, 16, 128, 512),
     W8A8 and bf16 (L2 flushed before each call);
+  * ``masks_grid`` and ``sqnr``: the sweep at batch 1, 8 and 32, and the SQNR of the masks' blocks.
+The result line carries, beside the ms/token of each mask and the W8A8 linears of ``kernels``:
   * ``roofline`` of the decode step's dominant kernel (the row-owning GEMV on bf16 weights, by
     share of device time) against the measured HBM copy bandwidth, with the lm_head GEMV beside it;
   * ``e2e``: decode through the public API with the token copied in from pinned host memory
@@ -914,6 +916,21 @@ def reference_line(args, times, n):
     }
 
 
+DETAILS = ("masks", "masks_grid", "batches", "kernels", "sqnr")
+
+
+def headline_and_details(line):
+    """The result line of stdout, a few kilobytes at most so that a log's tail holds it whole, and the
+    tables that go to stderr; of those the line keeps each mask's decode ms/token and the W8A8 linears."""
+    head = {k: v for k, v in line.items() if k not in DETAILS}
+    details = {k: line[k] for k in DETAILS if line.get(k) is not None}
+    table = (details.get("masks") or {}).get("rows")
+    if table:
+        head["masks_ms_per_token"] = {c["mask"]: c["ms_per_token"] for c in table}
+    head["w8a8_linears"] = {k: v for k, v in details.get("kernels", {}).items() if k.startswith(("linear_w8a8", "gemm_w8a8"))}
+    return head, {"details": details}
+
+
 def main():
     args = parse()
     if args.profile_workload:
@@ -959,7 +976,9 @@ def main():
             "kernels": res.get("kernels"),
             "sqnr": res.get("sqnr"), "setup_s": res["setup_s"],
         }
-        print(json.dumps(line))
+        head, details = headline_and_details(line)
+        print(json.dumps(details), file=sys.stderr, flush=True)
+        print(json.dumps(head))
     dist.close()
 
 

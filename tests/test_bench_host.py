@@ -1,5 +1,6 @@
 """Host-side logic of bench.py for N > 1 (replicas): the max-over-ranks reduction and the
 whole-job time-per-token figure, run as two gloo ranks on the CPU."""
+import json
 import os
 import socket
 
@@ -61,3 +62,14 @@ def test_decode_weight_bytes_of_the_masks():
     saved = 10 * 3 * 6912 * 1152 + 262144 * 1152
     assert bench.decode_weight_bytes(five, 0, 1) == bench.decode_weight_bytes(0, 0, 0) - saved
     assert bench.decode_weight_bytes(five, 0, 1) == pytest.approx(1.4586e9, rel=1e-4)
+
+
+def test_result_line_stays_short():
+    """Tables go to stderr: the result line fits a log's tail whole."""
+    rows = [{"mask": f"ffn {i} + lm", "ms_per_token": 0.57123, "ppl_delta": 0.1} for i in range(16)]
+    line = {"metric": bench.METRIC, "value": 0.57, "e2e": {"value": 0.6}, "masks": {"rows": rows}, "masks_grid": None,
+            "batches": {"x": [0.123456] * 400}, "kernels": {f"k{i}": {"us": 1.0} for i in range(60)}, "sqnr": {"db": [1.5] * 900}}
+    head, details = bench.headline_and_details(line)
+    assert len(json.dumps(head)) < 2000
+    assert head["value"] == 0.57 and head["e2e"] == {"value": 0.6} and len(head["masks_ms_per_token"]) == 16
+    assert set(details["details"]) == {"masks", "batches", "kernels", "sqnr"}
