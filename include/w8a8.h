@@ -423,8 +423,10 @@ w8a8_status w8a8_decode_gemv_plan(int weight_kind, int M, int N, int K, int gegl
  * without the fp16 code copy) for an [N, K] linear over M tokens.  out receives
  * W8A8_STREAM_PLAN_FIELDS ints: dp4a GEMV (1) or MMA streaming (0), whole 128-row groups per CTA,
  * dp4a token slots (0 on the MMA path), 8-token blocks per token group, tokens per group, token
- * groups, 128-row weight groups, k elements per stage, k chunks per row group, CTAs, CTAs per SM,
- * ring stages, stage bytes, dynamic shared memory bytes, partial-sum bytes.  W8A8_ERR_INVALID_ARG
+ * groups, 128-row weight groups, k elements per unit, k chunks per row group, CTAs, CTAs per SM,
+ * units that fit in the ring's room and the bytes of one with its token rows (the dp4a GEMV's ring stages; the
+ * MMA kernel cuts the same room into slots of one weight box, and keeps the token rows beside them when they
+ * are few), dynamic shared memory bytes, partial-sum bytes.  W8A8_ERR_INVALID_ARG
  * for a null out, M, N < 1, K < 16 or sms < 1. */
 #define W8A8_STREAM_PLAN_FIELDS 15
 w8a8_status w8a8_stream_gemm_plan(int int8_weights, int M, int N, int K, int sms, int* out);

@@ -17,7 +17,8 @@
 //    sliding window), takes the row maximum, p = exp(s - m), adds to the row sum (fp32) and writes P as
 //    fp16 into the swizzled shared-memory tile the second product reads.  m only moves when the
 //    maximum grew by more than 5.5 (p stays below e^5.5 = 245): O is then rescaled in tensor
-//    memory, rarely after the first tiles; any m gives the same quotient O / l;
+//    memory, rarely after the first tiles (the conditional rescaling that FlashAttention-4 published); any m
+//    gives the same quotient O / l;
 //  * a call with few tiles leaves most of the SMs idle, so the key tiles of a query block are split over the
 //    two CTAs of a cluster (tiles r, r + 2, ...), which exchange (m, l) and half of their O through
 //    distributed shared memory and finish 128 output dims each.

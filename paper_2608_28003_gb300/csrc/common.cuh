@@ -273,7 +273,8 @@ constexpr long long kWaitBudgetCycles = 4000000000LL;  // ~2 s at 2 GHz
 // Two fp32 values in one 64-bit register: each half of a packed operation is one IEEE operation,
 // rounded to nearest even.  A packed multiply feeding a packed add is contracted into one fused
 // operation whatever the rounding modifier says, so f2_mul adds a -0 that the compiler cannot know
-// (f2_neg_zero: gridDim.z is 1 in every launch); a b + (-0) is the rounded product, signs included.
+// (f2_neg_zero, for kernels whose gridDim.z is 1: the tcgen05 GEMM and the decode GEMV; not the attention
+// kernels, whose z is the batch); a b + (-0) is the rounded product, signs included.
 typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 f2_pack(float lo, float hi) {
   f32x2 r;

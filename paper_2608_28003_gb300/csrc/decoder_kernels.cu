@@ -239,8 +239,8 @@ __global__ void __launch_bounds__(kRowThreads) residual_norm_kernel(const uint16
   if (rq.inv_delta) row_quantize(rq, row, H, yv, red);
 }
 
-// The same step with a warp per row, for rows of at most 32 kWarpVec vectors and enough rows to fill the
-// GPU with such warps: a row's sums need shuffles only, and every lane has all of its loads in flight
+// The same step with a warp per row (its sums in another order than the block's), for rows of at most 32 kWarpVec
+// vectors and enough rows to fill the GPU with such warps: a row's sums need shuffles only, and every lane has all of its loads in flight
 // (with a block per row, 256 threads shared 144 vectors and met at eight barriers).  What bounds it is
 // the row's bytes (bf16 y in and a out, fp32 r in and out).  2048 rows of 1152: a 2048-token prefill
 // 4.25 -> 4.05 ms (52 launches); 640 rows 2.64 -> 2.58 ms.  Below 512 rows, which a block per row

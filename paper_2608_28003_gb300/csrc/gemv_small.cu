@@ -5,18 +5,17 @@
 // weight-streaming kernel splits such a layer's k sum over many CTAs and finishes it with a
 // partial-tile protocol through global memory; here every CTA owns R = 8 RW consecutive weight
 // rows over the full k range, so each sum ends inside its CTA:
-//  * one producer thread streams the CTA's rows through a shared-memory ring with 2-D TMA, starting
-//    before the preceding kernel has finished (weights do not depend on it).  A stage holds KS
-//    sub-slices of 512 bytes per row (each one or
-//    two unswizzled boxes of R rows x 256 elements), so that small-R calls still move enough bytes
-//    per pipeline round trip;
+//  * one producer thread streams the CTA's rows through a shared-memory ring with 2-D TMA, in all but a call's
+//    first launch starting before the preceding kernel has finished.  A stage holds KS sub-slices of 512
+//    bytes per row (each one or two unswizzled boxes of R rows x 256 elements), so that small-R calls still
+//    move enough bytes per pipeline round trip;
 //  * the consumer warps (8; 16 on the tensor-core paths of a grid with one CTA per SM) wait for
 //    the preceding kernel and stage the activations in shared
 //    memory, optionally computing them first from the decoder's residual step (residual add and
 //    the two RMSNorms, fused here instead of a separate launch).  The W8A8 path quantises them
 //    there, with the arithmetic of the stand-alone per-token quantiser (Eq. stx / xint8,
-//    smoothing of Eq. xhat-lmhead), so one launch does K1 and K3; at 9-16 tokens, and at 5-8 with a
-//    long K, the codes come from a launch of their own, since every CTA would repeat all that work;
+//    smoothing of Eq. xhat-lmhead), so one launch does K1 and K3; at 9-16 tokens, and on long rows at 5-8
+//    (separate_k1), the codes come from a launch of their own, since every CTA would repeat all that work;
 //  * warp w takes rows w, w + 8, ...; in every sub-slice lane l reads bytes 16 l .. 16 l + 15 of
 //    a row's 512 bytes (consecutive lanes read consecutive bytes: no bank conflicts);
 //  * INT8: four dp4a per 16 bytes and token, exact INT32 sums (Eq. gemm-final); bf16: fp32 FMAs,
@@ -531,12 +530,11 @@ __global__ void __launch_bounds__((CW + 1) * 32, CW == 8 ? 2 : 1)
           }
         }
       }
-    } else {
-      // 8 or 16 token slots: a warp (two of 16) per row, two short loops over its vectors, so that the
-      // rows run side by side and the code is small.  (All threads on all tokens, unrolled, was straight-line
-      // code that ran once per launch, and the warps waited for instructions: W8A8 1152 -> 6912 at 16
-      // tokens 13.8 us, now 11.1.)
-      constexpr int kRowWarps = CW >= MT ? CW / MT : 1;          // warps on one row
+    } else if constexpr (MT == 8) {  // (at 16 slots the codes always come from a launch before this one)
+      // Eight token slots: a warp (two of 16) per row, two short loops over its vectors, so that the rows run
+      // side by side and the code is small.  (All threads on all tokens, unrolled, was straight-line code that
+      // ran once per launch, and the warps waited for instructions: W8A8 FFN block at 8 tokens 20.6 us, so 20.0.)
+      constexpr int kRowWarps = CW / MT;  // warps on one row
       constexpr int kStep = 32 * kRowWarps;
       const ulonglong2* idl = reinterpret_cast<const ulonglong2*>(pre ? nullptr : constant(0, a.inv_delta));  // 1 / delta, two pairs each
       const f32x2 nz = f2_neg_zero();

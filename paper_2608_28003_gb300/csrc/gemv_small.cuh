@@ -40,7 +40,8 @@ struct SmallPlan {
 
 // The decoder's residual step in front of a decode linear, fused into the GEMV's prologue:
 // r_out = r_in + rmsnorm(y) * w_post, and the linear's input X = bf16(rmsnorm(r_out) * w_next),
-// with the arithmetic of the stand-alone residual-norm kernel (bit-identical results).  Every CTA
+// with the arithmetic of the stand-alone residual-norm kernel: at 1-4 token slots its sums too, bit for bit; at
+// 8 slots, a warp per row, and in the stand-alone form for long prompts the sums run in other orders.  Every CTA
 // computes the rows it needs; the first CTA writes r_out, so r_out must not alias r_in.
 struct ResNorm {
   const uint16_t* y;    // [M, K] bf16: the previous linear's output

@@ -76,7 +76,7 @@ __device__ __forceinline__ int row_perm(int g) {
   return kInt8 ? ((g >> 1) | ((g & 1) << 2)) : g;
 }
 
-// CTAs per SM: two for up to 16 tokens (registers allow it), else one.
+// CTAs per SM: two for up to 32 tokens (registers allow it), else one.
 template <int NB>
 struct Cps {
   static constexpr int value = NB <= 4 ? 2 : 1;

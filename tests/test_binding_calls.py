@@ -89,3 +89,29 @@ def test_optional_arguments(B):
     with pytest.raises(B.W8A8Error):
         B.ffn_block(B.FfnWeights(256, 512), B.W8A8_PREC_W8A8, x)  # no weights of that precision
     assert B.linear(q, x[:0]).shape == (0, 1024)
+
+
+@pytest.mark.gpu
+def test_descriptors_give_what_the_calls_give(B):
+    """The ctypes descriptors (c() of the weight classes) through the C ABI, as a caller of lib() uses them,
+    against the C module's own marshalling of the same objects."""
+    from ctypes import byref
+    dev = torch.device("cuda", 0)
+    x = torch.randn(8, 256, device=dev, generator=torch.Generator(dev).manual_seed(2)).to(torch.bfloat16)
+    q, qd = _qweight(B, 1024, 256, dev), _qweight(B, 256, 512, dev)
+    f8 = B.Fp8FfnWeights(256, 512, *(B.Fp8Weight(torch.randint(0, 0x70, t.wq.shape, dtype=torch.uint8, device=dev), t.s_w,
+                                                 t.delta, t.inv_delta) for t in (q, qd)))
+    f, hd = B.FfnWeights(256, 512, q, qd), B.HeadWeights(1024, 256, q)
+    ws = B.Workspace(dev).get(16 << 20)
+    y, st = torch.empty(8, 256, dtype=torch.bfloat16, device=dev), B._stream()
+    B._check("w8a8_ffn_block", B.lib().w8a8_ffn_block(byref(f.c()), B.W8A8_PREC_W8A8, B._p(x), 8, B._p(y), None, B._p(ws),
+                                                      ws.numel(), st))
+    assert torch.equal(B.ffn_block(f, B.W8A8_PREC_W8A8, x).view(torch.int16), y.view(torch.int16))
+    B._check("w8a8_fp8_ffn_block", B.lib().w8a8_fp8_ffn_block(byref(f8.c()), B._p(x), 8, B._p(y), None, B._p(ws),
+                                                              ws.numel(), st))
+    assert torch.equal(B.fp8_ffn_block(f8, x).view(torch.int16), y.view(torch.int16))
+    logits, top1 = torch.empty(8, 1024, device=dev), torch.empty(8, dtype=torch.int32, device=dev)
+    B._check("w8a8_lm_head", B.lib().w8a8_lm_head(byref(hd.c()), B.W8A8_PREC_W8A8, B._p(x), 8, B._p(logits), B._p(top1),
+                                                  B._p(ws), ws.numel(), st))
+    got = B.lm_head(hd, B.W8A8_PREC_W8A8, x)
+    assert torch.equal(got[0].view(torch.int32), logits.view(torch.int32)) and torch.equal(got[1], top1)
