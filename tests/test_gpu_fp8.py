@@ -103,7 +103,7 @@ def _oracle_linear(x32, prep):
 @pytest.mark.parametrize("M", [1, 2, 3, 8, 16, 64, 300])
 def test_fp8_linear_within_fp32_sum_bound(B, lin, M):
     """1-2 tokens: the decode GEMV with the codes widened to fp32 for FMAs; 3-16: the decode GEMV
-    on the tensor cores (e4m3 widened to fp16, mma.sync); K1 fused in both; more: K1 then the
+    on the tensor cores (e4m3 widened to fp16, mma.sync); K1 fused or a launch before it; more: K1 then the
     tcgen05 kind::f8f6f4 GEMM (single-CTA tiles, split-K at decode sizes)."""
     c, q, prep = lin
     Y, dbg = B.fp8_linear(q, cu(c["x"][:M]), debug=True)
